@@ -34,6 +34,7 @@
 // result does not depend on which other columns share the launch.
 #include "evc_internal.cuh"
 #include "evc_tridiag.cuh"
+#include "evc_dc.cuh"
 #include "evc_bulk.cuh"
 
 #include <cuda_bf16.h>
@@ -654,42 +655,45 @@ reorth_update_kernel(Run r, int i)
     if (threadIdx.x == 0) r.cnt_upd[ch] = 0;
 }
 
+// Whether shift s reads its quadratures at step i: at its last step and, under
+// a tolerance, from two steps before the first one the stop rule may take.
+__device__ __forceinline__ bool quad_needed(const Run& r, int s, int i)
+{
+    if (r.sdone[s]) return false;
+    return i >= r.skmax[s] || (r.stol[s] > 0.0 && i + 2 >= max(3, r.min_steps));
+}
+
 // Quadrature of every running column's J_i (Sec. 3, Eq. gauss_quad), or of
 // the extended J~_{2i-1} of the generalized averaged rule (Sec. 3.4,
-// Eq. GA_Tk) when r.ga is set.  One thread per Lanczos column; the
-// eigensolver scratch (3 x rule size per column) lives in shared memory.  In
-// shared mode one decomposition of the column's J_i serves every running
-// shift: the quadrature of shift s sums the weights of the Ritz values below
-// tau_s (J_i(A - tau I) = J_i(A) - tau I).
-__global__ void quad_kernel(Run r, int i)
+// Eq. GA_Tk) when r.ga is set.  One block per Lanczos column (evc_dc.cuh), in
+// shared memory.  In shared mode one decomposition of the column's J_i serves
+// every running shift: the quadrature of shift s sums the weights of the Ritz
+// values below tau_s (J_i(A - tau I) = J_i(A) - tau I).
+__global__ void __launch_bounds__(512) quad_kernel(Run r, int i)
 {
-    extern __shared__ double qs[];
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= r.ncol_real) return;
-    bool running;
+    extern __shared__ __align__(16) double qs[];
+    const int c = blockIdx.x;
+    int running = 0;
     if (r.shared) {
-        running = false;
-        for (int s = 0; s < r.S; ++s) running |= !r.sdone[s];
+        for (int s = threadIdx.x; s < r.S; s += blockDim.x) running |= quad_needed(r, s, i);
     } else {
-        running = !r.sdone[r.shift_of[c]];
+        running = quad_needed(r, r.shift_of[c], i);
     }
-    if (!running) return;
+    if (!__syncthreads_or(running)) return;
     const int k = r.kdone[c] ? min(r.kdone[c], i) : i;
-    const int nb = blockDim.x;
-    const int kk = r.ga ? 2 * r.kmax - 1 : r.kmax;
-    double* d = qs + threadIdx.x;
-    double* e = qs + (size_t)kk * nb + threadIdx.x;
-    double* z = qs + (size_t)2 * kk * nb + threadIdx.x;
-    const int kr = tridiag_fill(r.alpha + c, r.beta + c, r.ncol, k, r.ga != 0, d, e, nb);
-    const bool ok = tridiag_eig_inplace(d, e, z, nb, kr);
-    if (!ok) atomicExch(r.err, DERR_NUMERIC);
-    if (r.shared) {
-        for (int s = 0; s < r.S; ++s)
-            if (!r.sdone[s])
-                r.quad[(int64_t)s * r.m + c] =
-                    ok && c < r.m ? quadrature_below(d, z, nb, kr, (double)r.n, r.shifts[s]) : 0.0;
-    } else {
-        r.quad[c] = ok ? quadrature_below(d, z, nb, kr, (double)r.n, 0.0) : 0.0;
+    const int kr = r.ga && k > 1 ? 2 * k - 1 : k;
+    double* e = qs;
+    DcWork w = dc_carve(qs + ((kr + 1) & ~1), kr);
+    tridiag_fill(r.alpha + c, r.beta + c, r.ncol, k, r.ga != 0, w.d, e, threadIdx.x, blockDim.x);
+    __syncthreads();
+    int ex;
+    const bool ok = dc_solve(w, e, kr, ex);
+    if (!ok && threadIdx.x == 0) atomicExch(r.err, DERR_NUMERIC);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int s = warp; s < (r.shared ? r.S : 1); s += nw) {
+        if (r.shared && (r.sdone[s] || c >= r.m)) continue;
+        const double q = ok ? (double)r.n * dc_weight_below(w, kr, ex, r.shared ? r.shifts[s] : 0.0) : 0.0;
+        if (lane == 0) r.quad[r.shared ? (int64_t)s * r.m + c : c] = q;
     }
 }
 
@@ -869,22 +873,17 @@ cudaError_t launch_update(const Run& r, int i, cudaStream_t st)
 
 cudaError_t launch_finish(const Run& r, int i, cudaStream_t st)
 {
-    // The eigensolves are chains of dependent FP64 operations: spread the
-    // columns over all 152 SMs (few threads per block) so each one has an
-    // SM's FP64 pipes to itself; 3 scratch vectors per thread must fit in 96 KB.
-    const int kk = r.ga ? 2 * r.kmax - 1 : r.kmax;
-    int qb = 1;
-    while (qb < 32 && qb * 2 * 152 <= r.ncol_real) qb <<= 1;
-    while (qb > 1 && (size_t)qb * 3 * kk * sizeof(double) > 96 * 1024) qb >>= 1;
-    const size_t smem = (size_t)qb * 3 * kk * sizeof(double);
+    const int kr = r.ga && i > 1 ? 2 * i - 1 : i;
+    const size_t smem = dc_smem(kr) + (size_t)((kr + 1) & ~1) * sizeof(double);
     static std::atomic<uint64_t> attr{0};
-    const cudaError_t ea = smem_limit_once(attr, quad_kernel, 96 * 1024);
+    const int kmx = 2 * kMaxSteps - 1;
+    const cudaError_t ea = smem_limit_once(attr, quad_kernel, dc_smem(kmx) + (kmx + 1) * sizeof(double));
     if (ea != cudaSuccess) return ea;
     if (r.arnoldi) {
         const cudaError_t e = launch_arnoldi_quad(r, i, st);
         if (e != cudaSuccess) return e;
     } else {
-        quad_kernel<<<(r.ncol_real + qb - 1) / qb, qb, smem, st>>>(r, i);
+        quad_kernel<<<r.ncol_real, dc_threads(kr), smem, st>>>(r, i);
     }
     shift_kernel<<<r.S, kThreads, 0, st>>>(r, i);
     return cudaGetLastError();

@@ -1,9 +1,11 @@
 // evc_static.cu -- allocation-free batched Gauss quadrature (see
 // evc_gauss_quadrature_static in include/evc.h).  The eigensolver scratch
-// lives in one file-scope device array instead of caller- or library-
-// allocated memory, for callers that cannot allocate device memory.
+// lives in shared memory (one block per column) or, for many columns, in one
+// file-scope device array instead of caller- or library-allocated memory, for
+// callers that cannot allocate device memory.
 #include "evc_internal.cuh"
 #include "evc_tridiag.cuh"
+#include "evc_dc.cuh"
 #include "../../include/evc.h"
 
 #include <math_constants.h>
@@ -51,6 +53,35 @@ __global__ void static_quad_kernel(const double* alpha, const double* beta, cons
         if (status) atomicCAS(status, EVC_OK, EVC_ENUMERIC);
     }
     quad[c] = q;
+}
+
+// One block per column (evc_dc.cuh), all of it in shared memory.
+__global__ void __launch_bounds__(512)
+static_quad_block_kernel(const double* alpha, const double* beta, const int* kcol, int k, int ncol,
+                         double vnorm2, double* quad, int* status)
+{
+    extern __shared__ __align__(16) double qs[];
+    const int c = blockIdx.x;
+    const int kc = kcol ? kcol[c] : k;
+    if (kc < 1 || kc > k) {
+        if (threadIdx.x == 0) {
+            quad[c] = CUDART_NAN;
+            if (status) atomicCAS(status, EVC_OK, EVC_EINVAL);
+        }
+        return;
+    }
+    double* e = qs;
+    evc::DcWork w = evc::dc_carve(qs + ((kc + 1) & ~1), kc);
+    evc::tridiag_fill(alpha + c, beta + c, ncol, kc, false, w.d, e, threadIdx.x, blockDim.x);
+    __syncthreads();
+    int ex;
+    const bool ok = evc::dc_solve(w, e, kc, ex);
+    if (threadIdx.x >= 32) return;
+    const double q = ok ? vnorm2 * evc::dc_weight_below(w, kc, ex, 0.0) : CUDART_NAN;
+    if (threadIdx.x == 0) {
+        quad[c] = q;
+        if (!ok && status) atomicCAS(status, EVC_OK, EVC_ENUMERIC);
+    }
 }
 
 int say(char* buf, size_t len, int code, const char* msg)
@@ -105,8 +136,18 @@ extern "C" int evc_gauss_quadrature_static(const double* d_alpha, const double* 
             return say(errbuf, errlen, EVC_ECUDA, cudaGetErrorString(e));
         }
     }
-    static_quad_kernel<<<(ncol + 127) / 128, 128, 0, st>>>(d_alpha, d_beta, d_kcol, k, ncol,
-                                                            vnorm2, d_quad, scratch, d_status);
+    const size_t smem = evc::dc_smem(k) + (size_t)((k + 1) & ~1) * sizeof(double);   // at most 31 KB
+    // One block per column while the columns leave FP64 units idle; with more, a
+    // thread per column does less work in all.  Measured (thread | block): 64 x
+    // k = 40 3572 | 217 us, 4096 x k = 16 694 | 426, 16384 x k = 16 701 | 1501,
+    // 8192 x k = 32 about equal (2.5 ms); 4096 x k = 4 60 | 76, 2048 x k = 4
+    // about equal.
+    if (k >= 32 || ncol <= (k > 4 ? 4096 : 2048))
+        static_quad_block_kernel<<<ncol, evc::dc_threads(k), smem, st>>>(
+            d_alpha, d_beta, d_kcol, k, ncol, vnorm2, d_quad, d_status);
+    else
+        static_quad_kernel<<<(ncol + 127) / 128, 128, 0, st>>>(d_alpha, d_beta, d_kcol, k, ncol,
+                                                               vnorm2, d_quad, scratch, d_status);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return say(errbuf, errlen, EVC_ECUDA, cudaGetErrorString(e));
     return EVC_OK;

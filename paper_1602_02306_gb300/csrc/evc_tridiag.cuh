@@ -1,7 +1,7 @@
 // evc_tridiag.cuh -- Gauss quadrature of a symmetric tridiagonal matrix
 // (Sec. 3, Eq. gauss_quad): ||v||^2 sum_{theta_i < 0} z_i(1)^2 over the
-// eigenpairs (theta_i, z_i) of J_k.  Shared by the estimator's finish kernel
-// and the allocation-free quadrature entry point.
+// eigenpairs (theta_i, z_i) of J_k, one thread per matrix: the allocation-free
+// quadrature of many columns.  (One block per matrix: evc_dc.cuh.)
 #pragma once
 
 #include <cstdint>
@@ -105,29 +105,21 @@ __device__ inline double tridiag_quadrature_inplace(double* dp, double* ep, doub
     return quadrature_below(dp, zp, sstride, k, vnorm2, 0.0);
 }
 
-// Fill scratch with J_k (Gauss) or the extended J~_{2k-1} (GA); returns the
-// order of the filled matrix.  Layouts as in the two quadratures below.
-__device__ inline int tridiag_fill(const double* alpha, const double* beta, int64_t astride, int k,
-                                   bool ga, double* dp, double* ep, int64_t sstride)
+// Fill d[0..kk) and e[0..kk-1) with the diagonal and off-diagonal of J_k
+// (alpha[t*astride] = alpha_{t+1}, beta[t*astride] = beta_{t+1}, beta[0]
+// unused), or for the generalized averaged rule (Sec. 3.4, Eq. GA_Tk) with
+// those of the (2k-1) x (2k-1) tridiagonal with diagonal (alpha_1..alpha_k,
+// alpha_{k-1}..alpha_1) and off-diagonal (beta_2..beta_k, beta_{k+1},
+// beta_{k-1}..beta_2), which needs beta_{k+1}.  By nth threads, thread tid.
+__device__ inline void tridiag_fill(const double* alpha, const double* beta, int64_t astride, int k,
+                                    bool ga, double* d, double* e, int tid, int nth)
 {
-    if (!ga || k <= 1) {
-        for (int t = 0; t < k; ++t) {
-            dp[(int64_t)t * sstride] = alpha[(int64_t)t * astride];
-            ep[(int64_t)t * sstride] = t + 1 < k ? beta[(int64_t)(t + 1) * astride] : 0.0;
-        }
-        return k;
+    const int kk = ga && k > 1 ? 2 * k - 1 : k;
+    for (int t = tid; t < kk; t += nth) {
+        d[t] = alpha[(int64_t)(t < k ? t : 2 * k - 2 - t) * astride];
+        if (t + 1 < kk)
+            e[t] = beta[(int64_t)(t < k - 1 ? t + 1 : t == k - 1 ? k : 2 * k - 2 - t) * astride];
     }
-    const int kk = 2 * k - 1;
-    for (int t = 0; t < kk; ++t) {
-        const int a = t < k ? t : 2 * k - 2 - t;
-        dp[(int64_t)t * sstride] = alpha[(int64_t)a * astride];
-        double off = 0.0;
-        if (t < k - 1) off = beta[(int64_t)(t + 1) * astride];
-        else if (t == k - 1) off = beta[(int64_t)k * astride];
-        else if (t < kk - 1) off = beta[(int64_t)(2 * k - 2 - t) * astride];
-        ep[(int64_t)t * sstride] = off;
-    }
-    return kk;
 }
 
 // Gauss quadrature of J_k (Sec. 3, Eq. gauss_quad): alpha[t*astride] =
@@ -143,29 +135,6 @@ __device__ inline double tridiag_gauss_quadrature(const double* alpha, const dou
         ep[(int64_t)t * sstride] = t + 1 < k ? beta[(int64_t)(t + 1) * astride] : 0.0;
     }
     return tridiag_quadrature_inplace(dp, ep, zp, sstride, k, vnorm2);
-}
-
-// Generalized averaged Gauss quadrature (Sec. 3.4, Eq. GA_Tk): the same rule
-// on the (2k-1) x (2k-1) tridiagonal with diagonal (alpha_1..alpha_k,
-// alpha_{k-1}..alpha_1) and off-diagonal (beta_2..beta_k, beta_{k+1},
-// beta_{k-1}..beta_2).  Needs beta_{k+1} = beta[k*astride]; scratch of 2k-1
-// entries.  For k = 1 it is the Gauss rule.
-__device__ inline double tridiag_ga_quadrature(const double* alpha, const double* beta,
-                                               int64_t astride, int k, double vnorm2,
-                                               double* dp, double* ep, double* zp,
-                                               int64_t sstride)
-{
-    const int kk = 2 * k - 1;
-    for (int t = 0; t < kk; ++t) {
-        const int a = t < k ? t : 2 * k - 2 - t;               // mirrored alpha index
-        dp[(int64_t)t * sstride] = alpha[(int64_t)a * astride];
-        double off = 0.0;
-        if (t < k - 1) off = beta[(int64_t)(t + 1) * astride];            // beta_{t+2}
-        else if (t == k - 1) off = kk > 1 ? beta[(int64_t)k * astride] : 0.0;   // beta_{k+1}
-        else if (t < kk - 1) off = beta[(int64_t)(2 * k - 2 - t) * astride];   // mirrored
-        ep[(int64_t)t * sstride] = off;
-    }
-    return tridiag_quadrature_inplace(dp, ep, zp, sstride, kk, vnorm2);
 }
 
 }  // namespace evc
