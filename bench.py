@@ -170,7 +170,7 @@ def _roofline(evc, recs, peak, peak_kind, stencil_name="stencil_pass_kernel", W=
         tot = sum(v["ms"] for v in per_kind.values())
         roof["share_of_step"] = round(t / tot, 3) if tot > 0 else None
         return roof, per_kind
-    kernel = {"stencil": stencil_name, "csr": "csr_pass_kernel",
+    kernel = {"stencil": stencil_name, "csr": "csr_gather_kernel",
               "dots": "reorth_dots_kernel", "update": "reorth_update_kernel"}.get(name, name)
     ach = b / (t * 1e-3) / 1e9
     roof = {"bound": "hbm", "kernel": kernel, "achieved": round(ach, 1), "peak": peak,

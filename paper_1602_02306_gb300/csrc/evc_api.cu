@@ -271,6 +271,7 @@ size_t carve(const evc_ctx* c, int S, int m, int kmax, char* base, Run& r, void*
     r.basis_bf16 = c->basis_bf16;
     r.arnoldi = c->method == EVC_METHOD_ARNOLDI ? 1 : 0;
     r.hess = r.arnoldi ? D((size_t)kmax * (kmax + 1) / 2 * ncol) : nullptr;
+    r.gcopy = c->op == OP_CSR && uses_jac(c) && !r.tinv && !r.arnoldi;
     return off;
 }
 
@@ -983,7 +984,7 @@ int enqueue_all(evc_ctx* ctx, const Run& r, void* work, bool adaptive)
             rc = rec(ctx, EVC_K_REDUCE, i, colb * (2.0 * i + i * (i + 1) / 2), 0.0,
                      [&] { return launch_coef(r, i, st); });
         if (!rc)
-            rc = rec(ctx, EVC_K_UPDATE, i, 0.0, vchunk * (i + 2) + tw,
+            rc = rec(ctx, EVC_K_UPDATE, i, 0.0, vchunk * (i + 2 + (gather_copy(r, i + 1) ? 1 : 0)) + tw,
                      [&] { return launch_update<T>(r, i, st); });
         const bool last = (i == r.kmax);
         if (!rc && (adaptive || last))

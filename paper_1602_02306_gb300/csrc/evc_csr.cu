@@ -25,6 +25,7 @@ namespace {
 struct CArgs {
     CsrOp op;
     const void* x;          // slot i-1 of the basis (P_i)
+    const void* gx;         // its scaled copy m_r x_r (gather_copy), or null
     const void* pp;         // slot i-2 (P_{i-1}) or null
     void* out;              // slot i
     int64_t chunk_stride;
@@ -60,6 +61,52 @@ __device__ __forceinline__ Pack<T> ldg16(const T* p)
     return r;
 }
 
+// L2 policy of data that a pass reads or writes once: first to be evicted, so
+// that it does not push out the x rows, which are gathered again and again.
+__device__ __forceinline__ uint64_t policy_first()
+{
+    uint64_t p;
+    asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ int ld_once(const int* p, uint64_t pol)
+{
+    int v;
+    asm volatile("ld.global.nc.L2::cache_hint.b32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ float ld_once(const float* p, uint64_t pol)
+{
+    float v;
+    asm volatile("ld.global.nc.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ double ld_once(const double* p, uint64_t pol)
+{
+    double v;
+    asm volatile("ld.global.nc.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(p), "l"(pol));
+    return v;
+}
+template <typename T>
+__device__ __forceinline__ Pack<T> ld_once(const Pack<T>* p, uint64_t pol)
+{
+    uint4 t;
+    asm volatile("ld.global.nc.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=r"(t.x), "=r"(t.y), "=r"(t.z), "=r"(t.w) : "l"(p), "l"(pol));
+    Pack<T> r;
+    memcpy(&r, &t, 16);
+    return r;
+}
+template <typename T>
+__device__ __forceinline__ void st_once(Pack<T>* p, const Pack<T>& v, uint64_t pol)
+{
+    uint4 t;
+    memcpy(&t, &v, 16);
+    asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "r"(t.x),
+                 "r"(t.y), "r"(t.z), "r"(t.w), "l"(pol)
+                 : "memory");
+}
+
 // A group of LPR = CW / W lanes owns one row of one chunk; each lane holds W
 // consecutive columns (one 16-byte vector), so one gather instruction of the
 // warp fetches 32/LPR whole x rows.  Rows are visited in the order of
@@ -67,14 +114,12 @@ __device__ __forceinline__ Pack<T> ldg16(const T* p)
 // have similar lengths; each group broadcasts the row's (col, val) pairs from
 // its own lanes with warp shuffles.  UNI: every chunk's 32 columns belong to
 // one shift (m a multiple of 32, or one shift), so a gathered entry needs one
-// Jacobi scale, not one per column.  PM: PM_NONE, PM_JACOBI (row and column
-// scales m) or PM_TLEFT (row scale T = m^2 only; jac then holds m^2).
-template <typename T, int PM, bool UNI, int NT>
+// Jacobi scale, not one per column.  This kernel is the pass that scales the
+// gathered rows (PM_JACOBI without a scaled copy); csr_gather_kernel the others.
+template <typename T, bool UNI, int NT>
 __global__ void __launch_bounds__(NT)
 csr_pass_kernel(CArgs a)
 {
-    constexpr bool JAC = PM == PM_JACOBI;       // gathered rows scaled by m
-    constexpr bool ROWS = PM != PM_NONE;        // output rows scaled
     constexpr int W = 16 / sizeof(T);
     constexpr int LPR = CW / W;                 // lanes per row
     constexpr int RPW = 32 / LPR;               // rows per warp
@@ -93,7 +138,7 @@ csr_pass_kernel(CArgs a)
     const T* jr[NJ];
 #pragma unroll
     for (int w = 0; w < NJ; ++w)
-        jr[w] = ROWS ? static_cast<const T*>(a.jac) + (int64_t)a.shift_of[c0 + w] * n : nullptr;
+        jr[w] = static_cast<const T*>(a.jac) + (int64_t)a.shift_of[c0 + w] * n;
 
     const int64_t beg = valid ? a.op.row_ptr[row] : 0, end = valid ? a.op.row_ptr[row + 1] : 0;
     // the warp walks the longest of its rows; shorter rows contribute zeros
@@ -121,12 +166,12 @@ csr_pass_kernel(CArgs a)
             Pack<T> xa = ldg16(x + (int64_t)ca * CW + sub * W);
             Pack<T> xb = ldg16(x + (int64_t)cb * CW + sub * W);
             T ma = 1, mb = 1;
-            if (JAC && UNI) { ma = __ldg(jr[0] + ca); mb = __ldg(jr[0] + cb); }
+            if (UNI) { ma = __ldg(jr[0] + ca); mb = __ldg(jr[0] + cb); }
 #pragma unroll
             for (int w = 0; w < W; ++w) {
                 T sa = xa.v[w], sb = xb.v[w];
-                if (JAC && UNI) { sa = mul_rn(sa, ma); sb = mul_rn(sb, mb); }
-                if (JAC && !UNI) {
+                if (UNI) { sa = mul_rn(sa, ma); sb = mul_rn(sb, mb); }
+                if (!UNI) {
                     sa = mul_rn(sa, __ldg(jr[w] + ca));
                     sb = mul_rn(sb, __ldg(jr[w] + cb));
                 }
@@ -137,12 +182,12 @@ csr_pass_kernel(CArgs a)
             const int ca = __shfl_sync(0xffffffffu, mycol, grp * LPR + t);
             const T va = __shfl_sync(0xffffffffu, myval, grp * LPR + t);
             Pack<T> xa = ldg16(x + (int64_t)ca * CW + sub * W);
-            const T ma = JAC && UNI ? __ldg(jr[0] + ca) : (T)1;
+            const T ma = UNI ? __ldg(jr[0] + ca) : (T)1;
 #pragma unroll
             for (int w = 0; w < W; ++w) {
                 T sa = xa.v[w];
-                if (JAC && UNI) sa = mul_rn(sa, ma);
-                if (JAC && !UNI) sa = mul_rn(sa, __ldg(jr[w] + ca));
+                if (UNI) sa = mul_rn(sa, ma);
+                if (!UNI) sa = mul_rn(sa, __ldg(jr[w] + ca));
                 acc[w] = fma_rn(va, sa, acc[w]);
             }
         }
@@ -158,7 +203,7 @@ csr_pass_kernel(CArgs a)
     for (int w = 0; w < W; ++w) {
         const int c = c0 + w;
         T r = acc[w];
-        if (ROWS) r = mul_rn(r, __ldg(jr[UNI ? 0 : w] + row));
+        r = mul_rn(r, __ldg(jr[UNI ? 0 : w] + row));
         r = fma_rn(__ldg(dsh + (int64_t)a.shift_of[c] * n + row), cen.v[w], r);
         r = mul_rn(r, (T)a.insc[c]);
         if (pp) r = fma_rn(-(T)a.ppc[c], prev.v[w], r);
@@ -168,6 +213,103 @@ csr_pass_kernel(CArgs a)
     memcpy(&o, &res, 16);
     *reinterpret_cast<typename Vec16<T>::type*>(static_cast<T*>(a.out) + ch * a.chunk_stride +
                                                   row * CW + sub * W) = o;
+}
+
+// The pass on rows gathered as they are: PM_NONE, PM_TLEFT (output rows scaled
+// by T = m^2, which jac then holds) and, with PRE, PM_JACOBI from the scaled copy
+// of q_i.  Same ownership, same order of the sums and same roundings as above.
+// Bound by the latency of the gathers (128 or 256 bytes at random from L2 and
+// DRAM): all eight of a batch are in flight, the next batch of (col, val) pairs
+// is fetched meanwhile, and what the pass touches once leaves L2 first.  At least
+// 36 warps per SM: the registers that this leaves (56) hold the batch, and the
+// time no longer depends on the block size (two gathers in flight: 30 % slower;
+// eight without the bound: 1.18, 1.51 and 1.73 ms with 128, 64 and 256 threads).
+// (Past a row's end: its own row of x, times zero.)  ms per pass, before | now:
+//   64 columns x 2 shifts, power-law rows (mean 29), FP32, T^-1 process: 600k
+//   rows 1.44 | 1.00, 2M 4.85 | 4.41; Jacobi: 2M 5.28 | 4.60 and 0.16 more in the
+//   kernel that writes the copy, 600k 1.66 | 1.10, 30k (one row of 2000 entries
+//   is the critical path) 0.55 | 0.21; FP64 Jacobi 200k 2.49 | 1.42 (FP64 units:
+//   one operation per entry and column, before two).
+// 2M rows read 0.5 GB of structure and about 5 GB of x rows per chunk from DRAM
+// (the 256 MB of a chunk's x are twice L2) at 5 TB/s: what random 128-byte reads
+// reach there.  Slices of 16 or 8 columns of x, which fit L2, are no way out: 64
+// and 32-byte gathers took 6.5 and 10.7 ms per pass.
+template <typename T, int PM, int NT, bool PRE>
+__global__ void __launch_bounds__(NT, 36 * 32 / NT)
+csr_gather_kernel(CArgs a)
+{
+    static_assert(PM != PM_JACOBI || PRE, "the gathered rows are not scaled here");
+    constexpr int W = 16 / sizeof(T);
+    constexpr int LPR = CW / W;
+    constexpr int RPW = 32 / LPR;
+    constexpr int U = 8;                        // gathers in flight per lane
+    const int ch = blockIdx.y;
+    if (!a.chunk_active[ch]) return;
+    const int lane = threadIdx.x & 31;
+    const int grp = lane / LPR, sub = lane % LPR;
+    const int64_t slotrow = ((int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5)) * RPW + grp;
+    const int64_t n = a.op.n;
+    const bool valid = slotrow < n;
+    const int64_t row = valid ? (a.op.perm ? (int64_t)a.op.perm[slotrow] : slotrow) : 0;
+    const T* y = static_cast<const T*>(PRE ? a.gx : a.x) + ch * a.chunk_stride + sub * W;
+    const int64_t beg = valid ? a.op.row_ptr[row] : 0, len = valid ? a.op.row_ptr[row + 1] - beg : 0;
+    int64_t mx = len;
+#pragma unroll
+    for (int o = 16; o >= LPR; o >>= 1) mx = max(mx, (int64_t)__shfl_xor_sync(0xffffffffu, mx, o));
+    const uint64_t once = policy_first();
+    const int32_t* col = a.op.col + beg;
+    const T* val = static_cast<const T*>(a.op.val) + beg;
+    T acc[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) acc[w] = 0;
+    int ncol = (int)row;
+    T nval = 0;
+    if (sub < len) {
+        ncol = ld_once(col + sub, once);
+        nval = ld_once(val + sub, once);
+    }
+    for (int64_t k0 = 0; k0 < mx; k0 += LPR) {
+        const int mycol = ncol;
+        const T myval = mycol == (int)row ? (T)0 : nval;       // diagonal: from dsh
+        ncol = (int)row;
+        nval = 0;
+        if (k0 + LPR + sub < len) {
+            ncol = ld_once(col + k0 + LPR + sub, once);
+            nval = ld_once(val + k0 + LPR + sub, once);
+        }
+        const int cnt = (int)min((int64_t)LPR, mx - k0);
+#pragma unroll
+        for (int t = 0; t < LPR; t += U) {
+            if (t >= cnt) break;
+            Pack<T> xv[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                xv[u] = ldg16(y + (int64_t)__shfl_sync(0xffffffffu, mycol, grp * LPR + t + u) * CW);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const T v = __shfl_sync(0xffffffffu, myval, grp * LPR + t + u);
+#pragma unroll
+                for (int w = 0; w < W; ++w) acc[w] = fma_rn(v, xv[u].v[w], acc[w]);
+            }
+        }
+    }
+    if (!valid) return;
+    const int64_t at = ch * a.chunk_stride + row * CW + sub * W;
+    const Pack<T> cen = ldg16(static_cast<const T*>(a.x) + at);
+    Pack<T> prev, res;
+    if (a.pp) prev = ld_once(reinterpret_cast<const Pack<T>*>(static_cast<const T*>(a.pp) + at), once);
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+        const int c = ch * CW + sub * W + w;
+        const int64_t sr = (int64_t)a.shift_of[c] * n + row;
+        T r = acc[w];
+        if (PM != PM_NONE) r = mul_rn(r, __ldg(static_cast<const T*>(a.jac) + sr));
+        r = fma_rn(__ldg(static_cast<const T*>(a.dsh) + sr), cen.v[w], r);
+        r = mul_rn(r, (T)a.insc[c]);
+        if (a.pp) r = fma_rn(-(T)a.ppc[c], prev.v[w], r);
+        res.v[w] = r;
+    }
+    st_once(reinterpret_cast<Pack<T>*>(static_cast<T*>(a.out) + at), res, once);
 }
 
 }  // namespace
@@ -197,28 +339,23 @@ cudaError_t launch_csr_pass(const CsrOp& op, const Run& r, int i, int pmode, cud
     // every chunk's columns share one shift when m is a multiple of 32 (the
     // padding columns of the last chunk take the last shift) or S = 1
     const bool uni = r.S == 1 || r.m % CW == 0;
-    auto go = [&](auto pm_t, auto uni_t, auto nt_t) {
-        csr_pass_kernel<T, decltype(pm_t)::value, decltype(uni_t)::value, decltype(nt_t)::value>
-            <<<grid, decltype(nt_t)::value, 0, st>>>(a);
+    a.gx = gather_copy(r, i) ? basis + (int64_t)(i + 1) * r.slot_stride : nullptr;
+    auto launch = [&](auto nt_t) -> bool {
+        constexpr int NT = decltype(nt_t)::value;
+        if (pmode == PM_NONE) csr_gather_kernel<T, PM_NONE, NT, false><<<grid, NT, 0, st>>>(a);
+        else if (pmode == PM_TLEFT) csr_gather_kernel<T, PM_TLEFT, NT, false><<<grid, NT, 0, st>>>(a);
+        else if (pmode != PM_JACOBI) return false;
+        else if (a.gx) csr_gather_kernel<T, PM_JACOBI, NT, true><<<grid, NT, 0, st>>>(a);
+        else if (uni) csr_pass_kernel<T, true, NT><<<grid, NT, 0, st>>>(a);
+        else csr_pass_kernel<T, false, NT><<<grid, NT, 0, st>>>(a);
+        return true;
     };
-    using F = std::false_type;
-    using Tr = std::true_type;
-    auto by_nt = [&](auto pm_t, auto uni_t) -> bool {
-        switch (nt) {
-        case 128: go(pm_t, uni_t, std::integral_constant<int, 128>()); return true;
-        case 256: go(pm_t, uni_t, std::integral_constant<int, 256>()); return true;
-        case 512: go(pm_t, uni_t, std::integral_constant<int, 512>()); return true;
-        default: return false;
-        }
-    };
-    using PNone = std::integral_constant<int, PM_NONE>;
-    using PJac = std::integral_constant<int, PM_JACOBI>;
-    using PTl = std::integral_constant<int, PM_TLEFT>;
-    bool ok;
-    if (pmode == PM_NONE) ok = by_nt(PNone(), F());
-    else if (pmode == PM_JACOBI) ok = uni ? by_nt(PJac(), Tr()) : by_nt(PJac(), F());
-    else if (pmode == PM_TLEFT) ok = uni ? by_nt(PTl(), Tr()) : by_nt(PTl(), F());
-    else ok = false;
+    bool ok = false;
+    switch (nt) {
+    case 128: ok = launch(std::integral_constant<int, 128>()); break;
+    case 256: ok = launch(std::integral_constant<int, 256>()); break;
+    case 512: ok = launch(std::integral_constant<int, 512>()); break;
+    }
     if (!ok) return cudaErrorInvalidValue;
     return cudaGetLastError();
 }

@@ -125,7 +125,17 @@ struct Run {
     int basis_bf16;          // 1: basis vectors rounded to BF16 when stored (FP32 mode)
     int arnoldi;             // 1: Arnoldi process on T(A - sigma I) (Sec. 4)
     double* hess;            // [kmax(kmax+1)/2][ncol] Hessenberg columns (Arnoldi), or null
+    // CSR runs with Jacobi: the operator pass of step i gathers from a copy of
+    // q_i already scaled by the Jacobi m_r: an entry costs neither a second
+    // gather (of m_r) nor a second product per column.  The copy lies in slot
+    // i + 1 of the basis, which step i does not use yet (the last step has none
+    // and scales while it gathers); the kernel that stores q_i's final values
+    // writes it.
+    int gcopy;
 };
+
+// Whether step i gathers from the copy.
+__host__ __device__ inline bool gather_copy(const Run& r, int i) { return r.gcopy && i < r.kmax; }
 
 // Longest Arnoldi run: the quadrature keeps three k x k FP64 matrices in
 // shared memory (evc_arnoldi.cu): 195 KB at k = 90.

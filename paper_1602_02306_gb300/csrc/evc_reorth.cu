@@ -81,6 +81,9 @@ __global__ void init_probe_kernel(Run r)
         T v = (xh >> 63) ? (T)-1 : (T)1;
         if (r.tinv) v *= sqrt_rn(tdiag[(int64_t)r.shift_of[c] * r.n + row]);
         basis[ch * r.chunk_stride + row * CW + lane] = v;
+        if (gather_copy(r, 1))
+            basis[ch * r.chunk_stride + 2 * r.slot_stride + row * CW + lane] =
+                v * tdiag[(int64_t)r.shift_of[c] * r.n + row];
     }
 }
 
@@ -454,10 +457,12 @@ __global__ void reorth_coef_kernel(Run r, int i)
 // The producer streams, per row tile, the w tile and then every P_j tile;
 // consumer warp q owns rows q*RPW.. of the tile in registers and applies
 // every P_j stage to them, then writes the tile back.
-template <typename T, bool TW>
+// GC: also stores the scaled copy that the next operator pass gathers from.
+template <typename T, bool TW, bool GC>
 __global__ void __launch_bounds__(UTHREADS, 2)
 reorth_update_kernel(Run r, int i)
 {
+    static_assert(!(TW && GC), "the T^{-1} process gathers unscaled rows");
     constexpr int TR = USTAGE / (CW * (int)sizeof(T));   // rows per tile
     constexpr int RPW = TR / CWARPS;                      // rows per consumer warp
     const int ch = blockIdx.y, blk = blockIdx.x;
@@ -489,6 +494,8 @@ reorth_update_kernel(Run r, int i)
                            (int64_t)r.shift_of[ch * CW + (threadIdx.x & 31)] * r.n
                      : nullptr;
     const bool wuni = r.S == 1 || r.m % CW == 0;
+    T* gcopy = w + 2 * r.slot_stride + lane;
+    const T* gm = GC ? static_cast<const T*>(r.jac) + (int64_t)r.shift_of[ch * CW + lane] * r.n : nullptr;
     if (threadIdx.x == 0) {
         for (int s = 0; s < UNS; ++s) {
             mbar_init(&full[s], 1);
@@ -587,6 +594,7 @@ reorth_update_kernel(Run r, int i)
                     if (sizeof(T) == 4 && r.basis_bf16)
                         wv[rr] = (T)__bfloat162float(__float2bfloat16_rn((float)wv[rr]));
                     w[(row0 + row) * CW + lane] = wv[rr];
+                    if (GC) gcopy[(row0 + row) * CW] = wv[rr] * __ldg(gm + row0 + row);
                     if (TW && !wuni) d = __ldg(wt + row0 + row);
                     if (TW) nr += (RTy)(wv[rr] * d) * (RTy)wv[rr];
                     else nr += (RTy)wv[rr] * (RTy)wv[rr];
@@ -854,21 +862,23 @@ cudaError_t launch_coef(const Run& r, int i, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <typename T, bool TW>
+template <typename T, bool TW, bool GC>
 cudaError_t launch_update_w(const Run& r, int i, cudaStream_t st)
 {
     static std::atomic<uint64_t> attr{0};
     const cudaError_t e =
-        smem_limit_once(attr, reorth_update_kernel<T, TW>, update_smem<T>(kMaxSteps));
+        smem_limit_once(attr, reorth_update_kernel<T, TW, GC>, update_smem<T>(kMaxSteps));
     if (e != cudaSuccess) return e;
-    reorth_update_kernel<T, TW><<<dim3(r.nblk, r.nchunk), UTHREADS, update_smem<T>(i), st>>>(r, i);
+    reorth_update_kernel<T, TW, GC><<<dim3(r.nblk, r.nchunk), UTHREADS, update_smem<T>(i), st>>>(r, i);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_update(const Run& r, int i, cudaStream_t st)
 {
-    return r.tinv ? launch_update_w<T, true>(r, i, st) : launch_update_w<T, false>(r, i, st);
+    if (r.tinv) return launch_update_w<T, true, false>(r, i, st);
+    return gather_copy(r, i + 1) ? launch_update_w<T, false, true>(r, i, st)
+                                 : launch_update_w<T, false, false>(r, i, st);
 }
 
 cudaError_t launch_finish(const Run& r, int i, cudaStream_t st)
