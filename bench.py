@@ -319,11 +319,15 @@ def _measure(evc, W, args, stream, peak, peak_kind, steps, warmup, seed, tune=Tr
     launches = sum(1 for r in recs if not r[4])   # span records are not launches
     # the stencil class runs the patch kernel when the tuner chose 2 x 2 patches
     # (passes without Jacobi scaling, N even), the tiled kernel for patch 3
-    # (N a multiple of its 8 x 8 tile, else the patch kernel)
+    # (N a multiple of its 8 x 8 tile, else the patch kernel); the pairs of
+    # passes of a 7-point Chebyshev M in FP32 are one kernel whatever the shape
     sname = "stencil_pass_kernel"
     patch = tuning.get("stencil_patch") if tuning else _SHAPES["patch"]
     if W.kind == "stencil" and patch in (2, 3) and W.precond != "jacobi" and W.N % 2 == 0:
         sname = "stencil_tma_kernel" if patch == 3 and W.N % 8 == 0 else "stencil_patch_kernel"
+    if W.kind == "stencil" and W.precond == "cheb" and W.order == 2 and \
+            W.N % 2 == 0 and W.N >= 12 and not _CHEB_FORM[0]:
+        sname = "stencil_pair_kernel"
     roof, per_kind = _roofline(evc, recs, peak, peak_kind, sname, W)
     psteps = float(m * int(np.sum(st)))
     return ctx, {"ms": ms, "L": L, "steps_used": st, "quad": q, "clocks": clk, "roofline": roof,

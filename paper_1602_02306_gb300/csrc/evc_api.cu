@@ -691,6 +691,14 @@ int stencil(evc_ctx* ctx, const Run& r, int step, const StencilPass& p, int pmod
                [&] { return launch_stencil_pass<T>(ctx->sten, r, p, pmode, ctx->stream); });
 }
 
+// Both passes of a conjugate pair of roots in one launch (u is not stored).
+int stencil_pair(evc_ctx* ctx, const Run& r, int step, const StencilPass& first, const StencilPass& second)
+{
+    const double per = (double)r.n * CW * sizeof(float) * (2 + (second.pp ? 1 : 0));
+    return rec(ctx, EVC_K_STENCIL, step, 0.0, per,
+               [&] { return launch_stencil_pair(ctx->sten, r, first, second, ctx->stream); });
+}
+
 // y = p_d(K) x by Clenshaw's recurrence b_j = c_j x + 2 K~ b_{j+1} - b_{j+2},
 // y = c_0 x + K~ b_1 - b_2, K~ = (2K - (a+b)I)/(b-a).  Terms that are still
 // multiples of x are folded into the next pass, so degree d costs d passes;
@@ -719,11 +727,13 @@ int enqueue_cheb_factored(evc_ctx* ctx, const Run& r, int step, const void* x, i
         const evc_ctx::ChebFactor& F = ctx->cheb_fac[f];
         const bool last = f + 1 == nf;
         const double sg = last ? ctx->cheb_sign : 1.0;
-        void* dst = last ? out : Wb;
+        // one kernel for both passes of a pair where there is one: it reads its
+        // operand with a halo, so it never writes in place
+        const bool fused = F.pair && stencil_pair_eligible(ctx->sten, sizeof(T));
+        void* dst = last ? out : fused && cur == Wb ? Wa : Wb;
         const int64_t dst_cs = last ? out_cs : wcs;
-        StencilPass p{};
+        StencilPass p{}, pa{};
         if (F.pair) {
-            StencilPass pa{};
             pa.in = cur;
             pa.in_cs = cur_cs;
             pa.insc = cur_sc;
@@ -731,8 +741,10 @@ int enqueue_cheb_factored(evc_ctx* ctx, const Run& r, int step, const void* x, i
             pa.k0 = g * (c - F.re);
             pa.out = Wa;
             pa.out_cs = wcs;
-            int rc = stencil<T>(ctx, r, step, pa, PM_NONE);
-            if (rc) return rc;
+            if (!fused) {
+                int rc = stencil<T>(ctx, r, step, pa, PM_NONE);
+                if (rc) return rc;
+            }
             p.in = Wa;
             p.in_cs = wcs;
             p.k1 = sg * g;
@@ -757,7 +769,7 @@ int enqueue_cheb_factored(evc_ctx* ctx, const Run& r, int step, const void* x, i
             p.pp_cs = pp_cs;
             p.ppc = pp ? ppc : nullptr;
         }
-        int rc = stencil<T>(ctx, r, step, p, PM_NONE);
+        int rc = fused ? stencil_pair(ctx, r, step, pa, p) : stencil<T>(ctx, r, step, p, PM_NONE);
         if (rc) return rc;
         cur = dst;
         cur_cs = dst_cs;

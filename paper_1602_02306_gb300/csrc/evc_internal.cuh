@@ -212,6 +212,11 @@ template <typename T>
 cudaError_t launch_stencil_tma(const StencilOp& op, const StencilPass& p, const int* shift_of,
                                const double* sigma, const void* jac, const int* chunk_active,
                                int64_t n, int* err, int cn, int pmode, cudaStream_t st);
+// The two passes of a conjugate pair of roots of M = p_d(K) in one kernel
+// (evc_stencil_pair.cu): first x -> u, second u -> out; u is not stored.
+bool stencil_pair_eligible(const StencilOp& op, size_t tsize);
+cudaError_t launch_stencil_pair(const StencilOp& op, const Run& r, const StencilPass& first,
+                                const StencilPass& second, cudaStream_t st);
 // Arnoldi-type estimator (evc_arnoldi.cu)
 template <typename T>
 cudaError_t launch_row_scale(const Run& r, void* w, int64_t cs, cudaStream_t st);
