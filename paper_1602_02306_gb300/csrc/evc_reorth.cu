@@ -39,6 +39,7 @@
 
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 
 namespace evc {
@@ -164,6 +165,18 @@ __device__ __forceinline__ bool checked_bulk(void* dst, const void* src, uint32_
     return true;
 }
 
+// A consumer warp is done reading a stage.  The fence makes its reads complete
+// before the release: a load still queued behind another kernel's traffic on the
+// same SM would otherwise see the next copy, which a producer lane that waits for
+// this one barrier issues at once (seen in one of some ten counts that shared the
+// GPU with two others; the fence costs under 0.3% of either kernel).
+__device__ __forceinline__ void release(uint64_t* bar)
+{
+    fence_proxy_async_smem();
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+}
+
 template <typename T> struct Acc { typedef float run; };
 template <> struct Acc<double> { typedef double run; };
 
@@ -193,9 +206,21 @@ constexpr int UWARPS = CWARPS + NPROD;          // warps of the update kernel
 constexpr int UTHREADS = UWARPS * 32;           // threads of the update kernel
 static_assert(UNS % NPROD == 0, "a stage of the update ring must have one producer");
 
+// Basis vectors of part p of `parts` at step i: the groups p, p + parts, ... of JB.
+__host__ __device__ inline int dots_count(int i, int p, int parts)
+{
+    const int groups = (i + JB - 1) / JB, mine = (groups - p + parts - 1) / parts;
+    const bool last = mine > 0 && (groups - 1 - p) % parts == 0;       // has the last, short group
+    return mine * JB - (last ? groups * JB - i : 0);
+}
+
 // part_dot[ch][blk][j][lane]  = sum_{rows of blk} P_j[row][lane] * w[row][lane]
 // part_gram[ch][blk][j][lane] = sum_{rows of blk} P_j[row][lane] * P_{i-1}[row][lane]
-// for j < i.  Consumer warp q handles the basis vectors j = q, q+8, ...: it
+// for j < i.  With few row blocks the basis vectors of a row block are shared by
+// `parts` blocks (gridDim.z): part p takes the groups of JB vectors p, p + parts,
+// ...; every partial sum is still formed by one block in the same order, so the
+// split changes no bit.  Of its il vectors, numbered jl in the order of j,
+// consumer warp q handles jl = q, q+8, ...: it
 // holds the w and P_{i-1} tiles of the current row tile in registers and
 // owns the FP64 accumulators of its j's in shared memory, so every sum has a
 // fixed order (tiles in row order, FP32 runs of one tile in mixed mode).
@@ -214,13 +239,15 @@ __global__ void __launch_bounds__(DTHREADS, 2)
 reorth_dots_kernel(Run r, int i)
 {
     constexpr int TR = DSTAGE / (CW * (int)sizeof(T));   // rows per tile
-    const int ch = blockIdx.y, blk = blockIdx.x;
+    const int ch = blockIdx.y, blk = blockIdx.x, part = blockIdx.z, parts = gridDim.z;
     if (!r.chunk_active[ch]) return;
+    const int il = dots_count(i, part, parts);           // basis vectors of this block
+    auto jof = [&](int jl) { return (jl / JB * parts + part) * JB + jl % JB; };
     extern __shared__ __align__(128) unsigned char smem[];
     T* stage = reinterpret_cast<T*>(smem);                               // [DNS][TR*CW]
     T* wq = reinterpret_cast<T*>(smem + (size_t)DNS * DSTAGE);           // [2][2][TR*CW]
-    double* acc = reinterpret_cast<double*>(smem + (size_t)(DNS + 4) * DSTAGE);   // [2][i][CW]
-    uint64_t* full = reinterpret_cast<uint64_t*>(acc + (size_t)2 * i * CW);
+    double* acc = reinterpret_cast<double*>(smem + (size_t)(DNS + 4) * DSTAGE);   // [2][il][CW]
+    uint64_t* full = reinterpret_cast<uint64_t*>(acc + (size_t)2 * il * CW);
     uint64_t* empty = full + DNS;
     uint64_t* wqfull = empty + DNS;
     uint64_t* wqempty = wqfull + 2;
@@ -259,22 +286,26 @@ reorth_dots_kernel(Run r, int i)
         mbar_init_fence();
         s_fail = 0;
     }
-    for (int e = threadIdx.x; e < 2 * i * CW; e += blockDim.x) acc[e] = 0.0;
+    for (int e = threadIdx.x; e < 2 * il * CW; e += blockDim.x) acc[e] = 0.0;
     __syncthreads();
     typedef typename Acc<T>::run RTy;
     bool ok = true;
     if (warp >= CWARPS) {
-        // Producer p issues the items j = p, p + NPROD, ... -- the rings of the
-        // consumer warps cw = j % CWARPS with cw % NPROD == p, each ring in
-        // order -- so that NPROD threads issue bulk copies (one thread issues
-        // about one copy per quarter microsecond); producer 0 also issues the
-        // w and q_i tiles.
+        // Lane l of producer p feeds the rings of the consumer warps cw = p + NPROD
+        // (l + PL x), each in order; lane 0 of producer 0 also issues the w and q_i
+        // tiles.  FP32: one ring per lane, so that the waits and issues of the rings
+        // overlap (one thread issues about one copy per quarter microsecond; 2M rows,
+        // 128 columns: 75.6 -> 72.5 ms per 30 steps).  FP64 is bound by its consumers
+        // and loses to the polling lanes (200k rows: 89.8 -> 92.5 ms): one lane.
+        constexpr int RINGS = CWARPS / NPROD, PL = sizeof(T) == 4 ? RINGS : 1, RX = RINGS / PL;
         const int pw = warp - CWARPS;
         const bool weigh = PRODW && pw == 1;     // the whole warp weights the w, q tiles
-        if (lane == 0 || weigh) {
-            int64_t lastk[DNS];                  // last item issued into each stage
+        if (lane < PL || weigh) {
+            const int most = (il + CWARPS - 1) / CWARPS;     // items per tile of the first rings
+            int64_t done[RX];                    // items issued into each of this lane's rings
             int lastt[2] = {-1, -1};             // last tile issued into each w/q buffer
-            for (int s = 0; s < DNS; ++s) lastk[s] = -1;
+#pragma unroll
+            for (int x = 0; x < RX; ++x) done[x] = 0;
             for (int t = 0; t < ntile && ok; ++t) {
                 const int64_t row0 = r0 + (int64_t)t * TR;
                 const uint32_t bytes = (uint32_t)(min((int64_t)TR, r1 - row0) * CW * sizeof(T));
@@ -300,37 +331,41 @@ reorth_dots_kernel(Run r, int i)
                     fence_proxy_async_smem();
                     mbar_arrive(&wqready[b]);
                 }
-                if (lane == 0) {
-                    if (pw == 0) {
-                        // (warp 0 runs this loop on lane 0 alone: the break leaves it)
-                        if (t >= 2 && !(ok = mbar_wait(&wqempty[b], ((t >> 1) - 1) & 1))) break;
-                        lastt[b] = t;
-                        mbar_arrive_expect_tx(&wqfull[b], 2 * bytes);
-                        ok = checked_bulk(wq + (size_t)(2 * b) * TR * CW, w + row0 * CW, bytes,
-                                          &wqfull[b], lo, hi, r.err) &&
-                             checked_bulk(wq + (size_t)(2 * b + 1) * TR * CW, q + row0 * CW, bytes,
-                                          &wqfull[b], lo, hi, r.err);
-                    }
-                    for (int j = pw; j < i && ok; j += NPROD) {
-                        // k-th item of consumer warp cw lives in stage cw*NSW + k % NSW
-                        const int cw = j % CWARPS;
-                        const int64_t k = (int64_t)t * ((i - cw + CWARPS - 1) / CWARPS) + j / CWARPS;
+                if (pw == 0 && lane == 0) {
+                    if (t >= 2 && !(ok = mbar_wait(&wqempty[b], ((t >> 1) - 1) & 1))) break;
+                    lastt[b] = t;
+                    mbar_arrive_expect_tx(&wqfull[b], 2 * bytes);
+                    ok = checked_bulk(wq + (size_t)(2 * b) * TR * CW, w + row0 * CW, bytes, &wqfull[b], lo,
+                                      hi, r.err) &&
+                         checked_bulk(wq + (size_t)(2 * b + 1) * TR * CW, q + row0 * CW, bytes,
+                                      &wqfull[b], lo, hi, r.err);
+                }
+                for (int m = 0; m < most && ok && lane < PL; ++m) {
+#pragma unroll
+                    for (int x = 0; x < RX; ++x) {
+                        const int cw = pw + NPROD * (lane + PL * x), jl = cw + m * CWARPS;
+                        if (!ok || jl >= il) break;
+                        const int64_t k = done[x];
                         const int s = cw * NSW + (int)(k % NSW);
                         if (k >= NSW && !(ok = mbar_wait(&empty[s], ((k / NSW) - 1) & 1))) break;
-                        lastk[s] = k;
+                        done[x] = k + 1;
                         mbar_arrive_expect_tx(&full[s], bytes);
                         ok = checked_bulk(stage + (size_t)s * TR * CW,
-                                          P + (int64_t)j * r.slot_stride + row0 * CW, bytes,
-                                          &full[s], lo, hi, r.err);
+                                          P + (int64_t)jof(jl) * r.slot_stride + row0 * CW, bytes, &full[s],
+                                          lo, hi, r.err);
                     }
                 }
                 // the weighing warp leaves the loop as one
-                if (weigh) ok = __shfl_sync(0xffffffffu, ok, 0);
+                if (weigh) ok = __all_sync(0xffffffffu, ok);
             }
-            if (!ok) {
+            if (!ok && lane < PL) {
                 // let the copies already issued land before the block exits
-                for (int s = 0; s < DNS; ++s)
-                    if (lastk[s] >= 0) mbar_wait(&full[s], (lastk[s] / NSW) & 1);
+#pragma unroll
+                for (int x = 0; x < RX; ++x) {
+                    const int cw = pw + NPROD * (lane + PL * x);
+                    for (int64_t m = max((int64_t)0, done[x] - NSW); m < done[x]; ++m)
+                        mbar_wait(&full[cw * NSW + (int)(m % NSW)], (m / NSW) & 1);
+                }
                 for (int b = 0; b < 2; ++b)
                     if (lastt[b] >= 0) mbar_wait(&wqfull[b], (lastt[b] >> 1) & 1);
             }
@@ -355,11 +390,10 @@ reorth_dots_kernel(Run r, int i)
                     qv[rr] *= d;
                 }
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&wqempty[b]);
-            const int per = (i - warp + CWARPS - 1) / CWARPS;   // my items per tile
-            for (int j = warp; j < i; j += CWARPS) {
-                const int64_t k = (int64_t)t * per + j / CWARPS;
+            release(&wqempty[b]);
+            const int per = (il - warp + CWARPS - 1) / CWARPS;  // my items per tile
+            for (int jl = warp; jl < il; jl += CWARPS) {
+                const int64_t k = (int64_t)t * per + jl / CWARPS;
                 const int s = warp * NSW + (int)(k % NSW);
                 if (!(ok = mbar_wait_warp(&full[s], (k / NSW) & 1))) break;
                 const T* st = stage + (size_t)s * TR * CW + lane;
@@ -371,10 +405,9 @@ reorth_dots_kernel(Run r, int i)
                     a += pv * (RTy)wv[rr];
                     g += pv * (RTy)qv[rr];
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[s]);
-                acc[(size_t)j * CW + lane] += (double)a;
-                acc[(size_t)(i + j) * CW + lane] += (double)g;
+                release(&empty[s]);
+                acc[(size_t)jl * CW + lane] += (double)a;
+                acc[(size_t)(il + jl) * CW + lane] += (double)g;
             }
         }
     }
@@ -384,10 +417,10 @@ reorth_dots_kernel(Run r, int i)
         if (threadIdx.x == 0) atomicCAS(r.err, DERR_NONE, DERR_TIMEOUT);
         return;
     }
-    for (int e = threadIdx.x; e < i * CW; e += blockDim.x) {
-        const int64_t o = (((int64_t)ch * r.nblk + blk) * r.kmax + e / CW) * CW + (e % CW);
+    for (int e = threadIdx.x; e < il * CW; e += blockDim.x) {
+        const int64_t o = (((int64_t)ch * r.nblk + blk) * r.kmax + jof(e / CW)) * CW + (e % CW);
         r.part_dot[o] = acc[e];
-        r.part_gram[o] = acc[(size_t)i * CW + e];
+        r.part_gram[o] = acc[(size_t)il * CW + e];
     }
 }
 
@@ -410,11 +443,22 @@ reorth_reduce_kernel(Run r, int i)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ double sh[RW][CW], sg[RW][CW];
     double ah = 0.0, ag = 0.0;
-#pragma unroll 4
-    for (int b = warp; b < r.nblk; b += RW) {
-        const int64_t o = (((int64_t)ch * r.nblk + b) * r.kmax + j) * CW + lane;
-        ah += r.part_dot[o];
-        ag += r.part_gram[o];
+    // sixteen row blocks at a time in flight: all of a small problem's
+    constexpr int F = 16;
+    for (int b0 = warp; b0 < r.nblk; b0 += RW * F) {
+        double vh[F], vg[F];
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+            const int b = b0 + f * RW;
+            const int64_t o = (((int64_t)ch * r.nblk + b) * r.kmax + j) * CW + lane;
+            vh[f] = b < r.nblk ? r.part_dot[o] : 0.0;
+            vg[f] = b < r.nblk ? r.part_gram[o] : 0.0;
+        }
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+            ah += vh[f];
+            ag += vg[f];
+        }
     }
     sh[warp][lane] = ah;
     sg[warp][lane] = ag;
@@ -434,18 +478,28 @@ reorth_reduce_kernel(Run r, int i)
 }
 
 // c = h + (I - G) h;  g_j = c_j s_j multiplies the unnormalised P_j.
-// One thread per (column, j).
+// One thread per (column, j); the terms are added in the order of l (the rounding
+// of a g decides bits of every FP32 vector that follows), sixteen of them loaded at
+// a time: bound by the latency of those loads (four at a time: 15 us at i = 134,
+// two thirds of a step's small kernels).
 __global__ void reorth_coef_kernel(Run r, int i)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= r.ncol * i) return;
     const int c = t % r.ncol, j = t / r.ncol;
     if (!r.chunk_active[c / CW]) return;
+    constexpr int F = 16;
     double gh = 0.0;
-#pragma unroll 4
-    for (int l = 0; l < i; ++l) {
-        const double G = r.gram[(j >= l ? tri(j, l) : tri(l, j)) * r.ncol + c];
-        gh += G * r.hbuf[(int64_t)l * r.ncol + c];
+    for (int l0 = 0; l0 < i; l0 += F) {
+        double G[F], h[F];
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+            const int l = l0 + f;
+            G[f] = l < i ? r.gram[(j >= l ? tri(j, l) : tri(l, j)) * r.ncol + c] : 0.0;
+            h[f] = l < i ? r.hbuf[(int64_t)l * r.ncol + c] : 0.0;
+        }
+#pragma unroll
+        for (int f = 0; f < F; ++f) gh += G[f] * h[f];
     }
     const double hj = r.hbuf[(int64_t)j * r.ncol + c];
     r.g[(int64_t)j * r.ncol + c] = (2.0 * hj - gh) * r.scl[(int64_t)j * r.ncol + c];
@@ -456,7 +510,9 @@ __global__ void reorth_coef_kernel(Run r, int i)
 // w <- w - sum_{j<i} g_j P_j (in place, slot i); part_nrm = partial ||w||^2.
 // The producer streams, per row tile, the w tile and then every P_j tile;
 // consumer warp q owns rows q*RPW.. of the tile in registers and applies
-// every P_j stage to them, then writes the tile back.
+// every P_j stage to them, then writes the tile back.  In a small problem the
+// tiles of a row block are shared by uparts blocks (the FP32 runs of the norm stay
+// the same rows).
 // GC: also stores the scaled copy that the next operator pass gathers from.
 template <typename T, bool TW, bool GC>
 __global__ void __launch_bounds__(UTHREADS, 2)
@@ -465,7 +521,7 @@ reorth_update_kernel(Run r, int i)
     static_assert(!(TW && GC), "the T^{-1} process gathers unscaled rows");
     constexpr int TR = USTAGE / (CW * (int)sizeof(T));   // rows per tile
     constexpr int RPW = TR / CWARPS;                      // rows per consumer warp
-    const int ch = blockIdx.y, blk = blockIdx.x;
+    const int ch = blockIdx.y, blk = blockIdx.x;       // part blk % uparts of a row block
     if (!r.chunk_active[ch]) return;
     extern __shared__ __align__(128) unsigned char smem[];
     T* stage = reinterpret_cast<T*>(smem);                                // [UNS][TR*CW]
@@ -482,8 +538,17 @@ reorth_update_kernel(Run r, int i)
     for (int e = threadIdx.x; e < i * CW; e += blockDim.x)
         gs[e] = (T)r.g[(int64_t)(e / CW) * r.ncol + ch * CW + (e % CW)];
     int64_t r0, r1;
-    row_range(r.n, r.nblk, blk, r0, r1);
-    const int ntile = r1 > r0 ? (int)((r1 - r0 + TR - 1) / TR) : 0;
+    row_range(r.n, r.nblk, blk / r.uparts, r0, r1);
+    int ntile = r1 > r0 ? (int)((r1 - r0 + TR - 1) / TR) : 0;
+    {
+        // this part's tiles of the row block
+        const int p = blk % r.uparts, t0 = ntile * p / r.uparts, t1 = ntile * (p + 1) / r.uparts;
+        r1 = min(r1, r0 + (int64_t)t1 * TR);
+        r0 += (int64_t)t0 * TR;
+        ntile = t1 - t0;
+    }
+    const int nblk = r.nblk * r.uparts;
+    double* part_nrm = r.part_nrm + (int64_t)ch * nblk * CW;
     const T* P = static_cast<const T*>(r.basis) + ch * r.chunk_stride;
     T* w = static_cast<T*>(r.basis) + ch * r.chunk_stride + (int64_t)i * r.slot_stride;
     const void* lo = P;
@@ -513,45 +578,48 @@ reorth_update_kernel(Run r, int i)
     bool ok = true;
     double acc = 0.0;
     if (warp >= CWARPS) {
-        // Producer p issues the items with index = p (mod NPROD) -- the stages
-        // s = p (mod NPROD), each in order -- so that NPROD threads issue bulk
-        // copies; producer 0 also issues the w tiles.
+        // Lane l of producer p issues the items k = p + NPROD (l + PL x), in order.
+        // FP32: one stage per lane (see the dot kernel), and the next lane of producer
+        // 0 issues the w tiles; FP64: one lane, which issues a w tile before the
+        // tile's first item.
+        constexpr int PL = sizeof(T) == 4 ? UNS / NPROD : 1, STEP = NPROD * PL;
         const int pw = warp - CWARPS;
-        if (lane == 0) {
-            int64_t item = 0;
-            int64_t lastk[UNS];
-            int lastt[2] = {-1, -1};
-            for (int s = 0; s < UNS; ++s) lastk[s] = -1;
-            for (int t = 0; t < ntile && ok; ++t) {
+        auto issue_w = [&](int t) {
+            const int64_t row0 = r0 + (int64_t)t * TR;
+            const uint32_t bytes = (uint32_t)(min((int64_t)TR, r1 - row0) * CW * sizeof(T));
+            const int b = t & 1;
+            if (t >= 2 && !mbar_wait(&wempty[b], ((t >> 1) - 1) & 1)) return false;
+            mbar_arrive_expect_tx(&wfull[b], bytes);
+            return checked_bulk(wbuf + (size_t)b * TR * CW, w + row0 * CW, bytes, &wfull[b], lo, hi, r.err);
+        };
+        int tw = 0;                              // w tiles issued by this lane
+        if (lane < PL) {
+            int64_t k = pw + NPROD * lane;
+            int t = (int)(k / i), j = (int)(k % i);          // tile and basis vector of item k
+            for (; t < ntile && ok; k += STEP) {
+                if (PL == 1 && pw == 0)
+                    while (tw <= t && (ok = issue_w(tw))) ++tw;
+                const int s = (int)(k % UNS);
                 const int64_t row0 = r0 + (int64_t)t * TR;
                 const uint32_t bytes = (uint32_t)(min((int64_t)TR, r1 - row0) * CW * sizeof(T));
-                const int b = t & 1;
-                if (pw == 0) {
-                    if (t >= 2 && !(ok = mbar_wait(&wempty[b], ((t >> 1) - 1) & 1))) break;
-                    lastt[b] = t;
-                    mbar_arrive_expect_tx(&wfull[b], bytes);
-                    ok = checked_bulk(wbuf + (size_t)b * TR * CW, w + row0 * CW, bytes, &wfull[b],
-                                      lo, hi, r.err);
-                }
-                for (int j = 0; j < i && ok; ++j, ++item) {
-                    if ((int)(item % NPROD) != pw) continue;
-                    const int s = (int)(item % UNS);
-                    if (item >= UNS && !(ok = mbar_wait(&empty[s], ((item / UNS) - 1) & 1))) break;
-                    lastk[s] = item;
-                    mbar_arrive_expect_tx(&full[s], bytes);
-                    ok = checked_bulk(stage + (size_t)s * TR * CW,
-                                      P + (int64_t)j * r.slot_stride + row0 * CW, bytes, &full[s],
-                                      lo, hi, r.err);
-                }
+                if (!ok || (k >= UNS && !(ok = mbar_wait(&empty[s], ((k / UNS) - 1) & 1)))) break;
+                mbar_arrive_expect_tx(&full[s], bytes);
+                ok = checked_bulk(stage + (size_t)s * TR * CW, P + (int64_t)j * r.slot_stride + row0 * CW,
+                                  bytes, &full[s], lo, hi, r.err);
+                for (j += STEP; j >= i; j -= i) ++t;
             }
-            if (!ok) {
-                // let the copies already issued land before the block exits
-                for (int s = 0; s < UNS; ++s)
-                    if (lastk[s] >= 0) mbar_wait(&full[s], (lastk[s] / UNS) & 1);
-                for (int b = 0; b < 2; ++b)
-                    if (lastt[b] >= 0) mbar_wait(&wfull[b], (lastt[b] >> 1) & 1);
-            }
+            // (i = 1: the other producer has the last items, this one the last w tiles)
+            if (PL == 1 && pw == 0)
+                while (ok && tw < ntile && (ok = issue_w(tw))) ++tw;
+            // let the copies already issued land before the block exits
+            if (!ok)
+                for (int64_t m = max((int64_t)pw + NPROD * lane, k - UNS); m < k; m += STEP)
+                    mbar_wait(&full[m % UNS], (m / UNS) & 1);
+        } else if (PL > 1 && pw == 0 && lane == PL) {
+            for (; tw < ntile && ok; ++tw) ok = issue_w(tw);
         }
+        if (!ok)
+            for (int t = max(0, tw - 2); t < tw; ++t) mbar_wait(&wfull[t & 1], (t >> 1) & 1);
     } else {
         int64_t item = 0;
         for (int t = 0; t < ntile && ok; ++t) {
@@ -565,8 +633,7 @@ reorth_update_kernel(Run r, int i)
                 const int row = warp * RPW + rr;
                 wv[rr] = row < rows ? wbuf[(size_t)b * TR * CW + row * CW + lane] : (T)0;
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&wempty[b]);
+            release(&wempty[b]);
             for (int j = 0; j < i; ++j, ++item) {
                 const int s = (int)(item % UNS);
                 if (!(ok = mbar_wait_warp(&full[s], (item / UNS) & 1))) break;
@@ -575,8 +642,7 @@ reorth_update_kernel(Run r, int i)
 #pragma unroll
                 for (int rr = 0; rr < RPW; ++rr)
                     if (warp * RPW + rr < rows) wv[rr] -= gj * st[rr * CW];
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[s]);
+                release(&empty[s]);
             }
             if (!ok) break;
             RTy nr = 0;
@@ -614,21 +680,21 @@ reorth_update_kernel(Run r, int i)
         double sum = 0.0;
 #pragma unroll
         for (int qq = 0; qq < CWARPS; ++qq) sum += red[qq][lane];
-        r.part_nrm[((int64_t)ch * r.nblk + blk) * CW + lane] = sum;
+        part_nrm[(int64_t)blk * CW + lane] = sum;
     }
     // The last block of this chunk forms beta_{i+1}, the new scale s_i and the
     // breakdown test for the chunk's columns (no extra launch).
     __shared__ int s_last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&r.cnt_upd[ch], 1) == r.nblk - 1;
+    if (threadIdx.x == 0) s_last = atomicAdd(&r.cnt_upd[ch], 1) == nblk - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
     {
         double ps = 0.0;
-        for (int b = warp; b < r.nblk; b += UWARPS)
-            ps += r.part_nrm[((int64_t)ch * r.nblk + b) * CW + lane];
+        for (int b = warp; b < nblk; b += UWARPS)
+            ps += part_nrm[(int64_t)b * CW + lane];
         red[warp][lane] = ps;
     }
     __syncthreads();
@@ -839,7 +905,12 @@ cudaError_t launch_dots_w(const Run& r, int i, cudaStream_t st)
     static std::atomic<uint64_t> attr{0};
     const cudaError_t e = smem_limit_once(attr, reorth_dots_kernel<T, TW>, dots_smem<T>(kMaxSteps));
     if (e != cudaSuccess) return e;
-    reorth_dots_kernel<T, TW><<<dim3(r.nblk, r.nchunk), DTHREADS, dots_smem<T>(i), st>>>(r, i);
+    // two blocks per SM: where the row blocks do not give them, several blocks
+    // share a row block's vectors
+    const int groups = (i + JB - 1) / JB;
+    const int parts = std::min(groups, std::max(1, 2 * 152 / (r.nblk * r.nchunk)));
+    reorth_dots_kernel<T, TW><<<dim3(r.nblk, r.nchunk, parts), DTHREADS,
+                                dots_smem<T>((groups + parts - 1) / parts * JB), st>>>(r, i);
     return cudaGetLastError();
 }
 
@@ -857,8 +928,9 @@ cudaError_t launch_reduce(const Run& r, int i, cudaStream_t st)
 
 cudaError_t launch_coef(const Run& r, int i, cudaStream_t st)
 {
-    const int tot = r.ncol * i;
-    reorth_coef_kernel<<<(tot + 255) / 256, 256, 0, st>>>(r, i);
+    // few columns: small blocks, so that the loads spread over the SMs
+    const int tot = r.ncol * i, nth = tot >= 152 * 256 ? 256 : 64;
+    reorth_coef_kernel<<<(tot + nth - 1) / nth, nth, 0, st>>>(r, i);
     return cudaGetLastError();
 }
 
@@ -869,7 +941,7 @@ cudaError_t launch_update_w(const Run& r, int i, cudaStream_t st)
     const cudaError_t e =
         smem_limit_once(attr, reorth_update_kernel<T, TW, GC>, update_smem<T>(kMaxSteps));
     if (e != cudaSuccess) return e;
-    reorth_update_kernel<T, TW, GC><<<dim3(r.nblk, r.nchunk), UTHREADS, update_smem<T>(i), st>>>(r, i);
+    reorth_update_kernel<T, TW, GC><<<dim3(r.nblk * r.uparts, r.nchunk), UTHREADS, update_smem<T>(i), st>>>(r, i);
     return cudaGetLastError();
 }
 
