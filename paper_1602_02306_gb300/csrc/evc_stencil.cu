@@ -18,6 +18,7 @@
 // in flight are held by shared memory rather than registers.  The pass is
 // HBM-bound: it streams the operand once and the pointwise operands once.
 #include "evc_internal.cuh"
+#include "evc_stencil_fold.cuh"
 
 #include <cstring>
 
@@ -106,12 +107,14 @@ stencil_pass_kernel(KArgs a)
     Pack<T>* slots = reinterpret_cast<Pack<T>*>(st_raw);      // [DEPTH+1][NL][STH]
     // per-column constants of this chunk, shared by the block
     __shared__ Pack<T> s_sig[LPP], s_insc[LPP], s_a0s[LPP], s_ppc[LPP];
+    __shared__ Fold64<LPP> s_f;
     __shared__ int s_shift[CW];
     if (threadIdx.x < CW) {
         const int c = ch * CW + threadIdx.x;
         const int l = threadIdx.x / W, w = threadIdx.x % W;
         s_sig[l].v[w] = VS ? (T)a.sigma[c] : (T)0;
         s_insc[l].v[w] = a.p.insc ? (T)a.p.insc[c] : (T)1;
+        if constexpr (sizeof(T) == 8) s_f.set(l, w, a.p, a.op, s_insc[l].v[w], s_sig[l].v[w]);
         s_a0s[l].v[w] = (T)(a.p.a0 * (a.p.xs ? a.p.xs[c] : 1.0));
         s_ppc[l].v[w] = PP ? (T)a.p.ppc[c] : (T)0;
         s_shift[threadIdx.x] = ROWS ? a.shift_of[c] : 0;
@@ -229,6 +232,17 @@ stencil_pass_kernel(KArgs a)
         Pack<T> res;
 #pragma unroll
         for (int w = 0; w < W; ++w) {
+            if constexpr (sizeof(T) == 8) {
+                const T s1 = nb[0].v[w] + nb[1].v[w] + nb[2].v[w] + nb[3].v[w] + win[R - 1].v[w] +
+                             win[R + 1].v[w];
+                T s2 = 0;
+                if (R == 2)
+                    s2 = nb[4 % (4 * R)].v[w] + nb[5 % (4 * R)].v[w] + nb[6 % (4 * R)].v[w] +
+                         nb[7 % (4 * R)].v[w] + win[0].v[w] + win[2 * R].v[w];
+                res.v[w] = s_f.template apply<R, VS>(lane, w, s1, s2, win[R].v[w], insc.v[w], vp);
+                if (ROWS) res.v[w] *= mp[w];
+                continue;
+            }
             T off = c1 * (nb[0].v[w] + nb[1].v[w] + nb[2].v[w] + nb[3].v[w] +
                           win[R - 1].v[w] + win[R + 1].v[w]);
             if (R == 2)
@@ -331,12 +345,14 @@ stencil_patch_kernel(KArgs a)
     extern __shared__ __align__(16) unsigned char st_raw[];
     Pack<T>* slots = reinterpret_cast<Pack<T>*>(st_raw);      // [DEPTHP+1][NL][STP]
     __shared__ Pack<T> s_sig[LPP], s_insc[LPP], s_a0s[LPP], s_ppc[LPP];
+    __shared__ Fold64<LPP> s_f;
     __shared__ int s_shift[CW];
     if (threadIdx.x < CW) {
         const int c = ch * CW + threadIdx.x;
         const int l = threadIdx.x / W, w = threadIdx.x % W;
         s_sig[l].v[w] = VS ? (T)a.sigma[c] : (T)0;
         s_insc[l].v[w] = a.p.insc ? (T)a.p.insc[c] : (T)1;
+        if constexpr (sizeof(T) == 8) s_f.set(l, w, a.p, a.op, s_insc[l].v[w], s_sig[l].v[w]);
         s_a0s[l].v[w] = (T)(a.p.a0 * (a.p.xs ? a.p.xs[c] : 1.0));
         s_ppc[l].v[w] = PP ? (T)a.p.ppc[c] : (T)0;
         s_shift[threadIdx.x] = ROWS ? a.shift_of[c] : 0;
@@ -468,6 +484,18 @@ stencil_patch_kernel(KArgs a)
                 Pack<T> res;
 #pragma unroll
                 for (int w = 0; w < W; ++w) {
+                    if constexpr (sizeof(T) == 8) {
+                        const T s1 = nbv(-1, 0).v[w] + nbv(1, 0).v[w] + nbv(0, -1).v[w] + nbv(0, 1).v[w] +
+                                     win[R - 1][pp_].v[w] + win[R + 1][pp_].v[w];
+                        T s2 = 0;
+                        if (R == 2)
+                            s2 = nbv(-2, 0).v[w] + nbv(2, 0).v[w] + nbv(0, -2).v[w] + nbv(0, 2).v[w] +
+                                 win[0][pp_].v[w] + win[2 * R][pp_].v[w];
+                        res.v[w] = s_f.template apply<R, VS>(lane, w, s1, s2, win[R][pp_].v[w], insc.v[w], vp);
+                        if (ROWS)
+                            res.v[w] *= __ldg(jac + (int64_t)s_shift[lane * W + w] * n + cxy[pp_] + rowz);
+                        continue;
+                    }
                     T off = c1 * (nbv(-1, 0).v[w] + nbv(1, 0).v[w] + nbv(0, -1).v[w] +
                                   nbv(0, 1).v[w] + win[R - 1][pp_].v[w] + win[R + 1][pp_].v[w]);
                     if (R == 2)

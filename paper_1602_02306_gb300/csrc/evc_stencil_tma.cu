@@ -25,6 +25,7 @@
 // its own copies in flight before it exits.
 #include "evc_internal.cuh"
 #include "evc_bulk.cuh"
+#include "evc_stencil_fold.cuh"
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -208,12 +209,14 @@ stencil_tma_kernel(const __grid_constant__ TmaMaps maps, const TmaArgs a)
     __shared__ uint64_t fullA[LA], fullB[LB], emptyA[LA], emptyB[LB];
     __shared__ int s_fail, s_lastA, s_lastB;
     __shared__ Pack<T> s_sig[LPP], s_insc[LPP], s_a0s[LPP], s_ppc[LPP];
+    __shared__ Fold64<LPP> s_f;
     __shared__ int s_shift[CW];
     if (threadIdx.x < CW) {
         const int c = ch * CW + threadIdx.x;
         const int l = threadIdx.x / W, w = threadIdx.x % W;
         s_sig[l].v[w] = VS ? (T)a.sigma[c] : (T)0;
         s_insc[l].v[w] = a.p.insc ? (T)a.p.insc[c] : (T)1;
+        if constexpr (sizeof(T) == 8) s_f.set(l, w, a.p, a.op, s_insc[l].v[w], s_sig[l].v[w]);
         s_a0s[l].v[w] = (T)(a.p.a0 * (a.p.xs ? a.p.xs[c] : 1.0));
         s_ppc[l].v[w] = PP ? (T)a.p.ppc[c] : (T)0;
         s_shift[threadIdx.x] = ROWS ? a.shift_of[c] : 0;
@@ -383,6 +386,18 @@ stencil_tma_kernel(const __grid_constant__ TmaMaps maps, const TmaArgs a)
                     Pack<T> res;
 #pragma unroll
                     for (int w = 0; w < W; ++w) {
+                        if constexpr (sizeof(T) == 8) {
+                            const T s1 = xm1.v[w] + xp1.v[w] + ym1.v[w] + yp1.v[w] + win[R - 1][pp_].v[w] +
+                                         win[R + 1][pp_].v[w];
+                            T s2 = 0;
+                            if (R == 2)
+                                s2 = xm2.v[w] + xp2.v[w] + ym2.v[w] + yp2.v[w] + win[0][pp_].v[w] +
+                                     win[2 * R][pp_].v[w];
+                            res.v[w] = s_f.template apply<R, VS>(lane, w, s1, s2, win[R][pp_].v[w], insc.v[w], vp);
+                            if (ROWS)
+                                res.v[w] *= __ldg(jac + (int64_t)s_shift[lane * W + w] * n + cxy[pp_] + rowz);
+                            continue;
+                        }
                         T off = c1 * (xm1.v[w] + xp1.v[w] + ym1.v[w] +
                                       yp1.v[w] + win[R - 1][pp_].v[w] + win[R + 1][pp_].v[w]);
                         if (R == 2)
