@@ -167,14 +167,16 @@ int choose_nblk(int64_t n, int rows)
     return (int)std::max<int64_t>(1, std::min<int64_t>((n + rows - 1) / rows, 65535));
 }
 
-// Blocks of the update kernel per row block, by n alone for the same reason: a
-// small problem's 64 row blocks per chunk leave SMs idle (in the dot kernel the
-// blocks of a row block share its vectors instead, which changes no sum).  127^2
-// rows: 9.6 -> 8.5 ms per 134 steps, 40^3: 1.40 -> 1.16 ms per 24; three blocks and
-// more cost more than they give.
-int choose_uparts(int64_t n, int nblk)
+// Segments of a row block with a partial norm each, which the blocks of the update
+// kernel share: by n and the row blocks alone for the same reason.  Three (one or
+// three blocks) for long row blocks; two for short ones, whose pipelines would not
+// pay more blocks; one where the row blocks are many anyway, so that the block which
+// adds the partial norms up stays short (2M rows keep their 579 row blocks).  At most
+// twice nblk_max / nblk: see part_nrm.
+int choose_useg(int64_t n, int nblk)
 {
-    return n < (int64_t)64 * 3456 ? std::min(2, std::max(1, reorth_max_blocks(n) / nblk)) : 1;
+    if (nblk >= 512) return 1;
+    return n >= (int64_t)2048 * nblk && 2 * reorth_max_blocks(n) >= 3 * nblk ? 3 : 2;
 }
 
 struct Layout {
@@ -233,7 +235,7 @@ size_t carve(const evc_ctx* c, int S, int m, int kmax, char* base, Run& r, void*
     r.Sop = Sop;
     r.nchunk = nchunk;
     r.nblk = nblk;
-    r.uparts = choose_uparts(c->n, nblk);
+    r.useg = choose_useg(c->n, nblk);
     r.slot_stride = c->n * CW;
     r.chunk_stride = (int64_t)(kmax + 1) * c->n * CW;
     r.basis = take((size_t)nchunk * (kmax + 1) * vec);
@@ -273,7 +275,10 @@ size_t carve(const evc_ctx* c, int S, int m, int kmax, char* base, Run& r, void*
     r.part_gram = D((size_t)nchunk * nblk_max * kmax * CW);
     r.hbuf = D((size_t)kmax * ncol);
     r.gram = D((size_t)kmax * (kmax + 1) / 2 * ncol);
-    r.part_nrm = D((size_t)nchunk * nblk_max * CW);
+    // the partial norms take the place of the step's partial dot products and Gram
+    // entries (one array after the other, 2 kmax nblk_max rows per chunk), already
+    // summed when the norms are formed
+    r.part_nrm = r.part_dot;
     r.err = I(1);
     r.seed = reinterpret_cast<uint64_t*>(take(8));
     r.breakdown_rel = c->precision == EVC_FP64 ? 1e-12 : 1e-6;

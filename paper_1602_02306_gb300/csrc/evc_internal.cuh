@@ -73,7 +73,7 @@ struct Run {
     double* opshift;         // [Sop] shift of the operator the columns run on
     int nchunk;
     int nblk;                // row blocks per chunk in the reorth kernels
-    int uparts;              // blocks of the update kernel per row block
+    int useg;                // segments of a row block in the update kernel
     int64_t slot_stride;     // n*CW elements
     int64_t chunk_stride;    // (kmax+1)*n*CW elements
     void* basis;             // T[nchunk][kmax+1][n][CW]
@@ -107,7 +107,7 @@ struct Run {
     double* part_gram;       // [nchunk][nblk][kmax][CW]  partial P_j . P_{i-1}
     double* hbuf;            // [kmax][ncol]  h_j = q_j . w of the current step
     double* gram;            // [kmax(kmax+1)/2][ncol]  G_ab = q_a . q_b, a >= b
-    double* part_nrm;        // [nchunk][nblk*uparts][CW]
+    double* part_nrm;        // [nchunk][nblk*useg][CW]
     void* jac;               // T[Sop][n]  Jacobi scales m_r (or m_r^2 = T in T^{-1} mode)
     void* dsh;               // T[Sop][n]  CSR contexts: the diagonal of the shifted operator,
                              //   (a_rr - sigma) m_r^2 (Lanczos with Jacobi) or a_rr - sigma,

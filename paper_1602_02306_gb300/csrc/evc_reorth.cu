@@ -510,9 +510,9 @@ __global__ void reorth_coef_kernel(Run r, int i)
 // w <- w - sum_{j<i} g_j P_j (in place, slot i); part_nrm = partial ||w||^2.
 // The producer streams, per row tile, the w tile and then every P_j tile;
 // consumer warp q owns rows q*RPW.. of the tile in registers and applies
-// every P_j stage to them, then writes the tile back.  In a small problem the
-// tiles of a row block are shared by uparts blocks (the FP32 runs of the norm stay
-// the same rows).
+// every P_j stage to them, then writes the tile back.  The tiles of a row block
+// form r.useg segments with a partial norm each, and gridDim.x / nblk blocks share
+// them (launch_update_w): the split changes no bit.
 // GC: also stores the scaled copy that the next operator pass gathers from.
 template <typename T, bool TW, bool GC>
 __global__ void __launch_bounds__(UTHREADS, 2)
@@ -521,7 +521,8 @@ reorth_update_kernel(Run r, int i)
     static_assert(!(TW && GC), "the T^{-1} process gathers unscaled rows");
     constexpr int TR = USTAGE / (CW * (int)sizeof(T));   // rows per tile
     constexpr int RPW = TR / CWARPS;                      // rows per consumer warp
-    const int ch = blockIdx.y, blk = blockIdx.x;       // part blk % uparts of a row block
+    const int parts = gridDim.x / r.nblk;
+    const int ch = blockIdx.y, blk = blockIdx.x / parts, part = blockIdx.x % parts;
     if (!r.chunk_active[ch]) return;
     extern __shared__ __align__(128) unsigned char smem[];
     T* stage = reinterpret_cast<T*>(smem);                                // [UNS][TR*CW]
@@ -538,17 +539,15 @@ reorth_update_kernel(Run r, int i)
     for (int e = threadIdx.x; e < i * CW; e += blockDim.x)
         gs[e] = (T)r.g[(int64_t)(e / CW) * r.ncol + ch * CW + (e % CW)];
     int64_t r0, r1;
-    row_range(r.n, r.nblk, blk / r.uparts, r0, r1);
-    int ntile = r1 > r0 ? (int)((r1 - r0 + TR - 1) / TR) : 0;
-    {
-        // this part's tiles of the row block
-        const int p = blk % r.uparts, t0 = ntile * p / r.uparts, t1 = ntile * (p + 1) / r.uparts;
-        r1 = min(r1, r0 + (int64_t)t1 * TR);
-        r0 += (int64_t)t0 * TR;
-        ntile = t1 - t0;
-    }
-    const int nblk = r.nblk * r.uparts;
-    double* part_nrm = r.part_nrm + (int64_t)ch * nblk * CW;
+    row_range(r.n, r.nblk, blk, r0, r1);
+    // this block's segments s0 .. s1 - 1 of the row block, tiles t0 .. t0 + ntile - 1
+    const int ntb = r1 > r0 ? (int)((r1 - r0 + TR - 1) / TR) : 0;
+    const int s0 = r.useg * part / parts, s1 = r.useg * (part + 1) / parts;
+    const int t0 = ntb * s0 / r.useg, ntile = ntb * s1 / r.useg - t0;
+    r1 = min(r1, r0 + (int64_t)(t0 + ntile) * TR);
+    r0 += (int64_t)t0 * TR;
+    const int nnrm = r.nblk * r.useg;
+    double* part_nrm = r.part_nrm + (int64_t)ch * nnrm * CW;
     const T* P = static_cast<const T*>(r.basis) + ch * r.chunk_stride;
     T* w = static_cast<T*>(r.basis) + ch * r.chunk_stride + (int64_t)i * r.slot_stride;
     const void* lo = P;
@@ -576,7 +575,6 @@ reorth_update_kernel(Run r, int i)
     __syncthreads();
     typedef typename Acc<T>::run RTy;
     bool ok = true;
-    double acc = 0.0;
     if (warp >= CWARPS) {
         // Lane l of producer p issues the items k = p + NPROD (l + PL x), in order.
         // FP32: one stage per lane (see the dot kernel), and the next lane of producer
@@ -622,79 +620,93 @@ reorth_update_kernel(Run r, int i)
             for (int t = max(0, tw - 2); t < tw; ++t) mbar_wait(&wfull[t & 1], (t >> 1) & 1);
     } else {
         int64_t item = 0;
-        for (int t = 0; t < ntile && ok; ++t) {
-            const int64_t row0 = r0 + (int64_t)t * TR;
-            const int rows = (int)min((int64_t)TR, r1 - row0);
-            const int b = t & 1;
-            if (!(ok = mbar_wait_warp(&wfull[b], (t >> 1) & 1))) break;
-            T wv[RPW];
+        int t = 0;
+        for (int seg = s0; seg < s1; ++seg) {
+            double acc = 0.0;
+            for (const int te = ntb * (seg + 1) / r.useg - t0; t < te && ok; ++t) {
+                const int64_t row0 = r0 + (int64_t)t * TR;
+                const int rows = (int)min((int64_t)TR, r1 - row0);
+                const int b = t & 1;
+                if (!(ok = mbar_wait_warp(&wfull[b], (t >> 1) & 1))) break;
+                T wv[RPW];
 #pragma unroll
-            for (int rr = 0; rr < RPW; ++rr) {
-                const int row = warp * RPW + rr;
-                wv[rr] = row < rows ? wbuf[(size_t)b * TR * CW + row * CW + lane] : (T)0;
-            }
-            release(&wempty[b]);
-            for (int j = 0; j < i; ++j, ++item) {
-                const int s = (int)(item % UNS);
-                if (!(ok = mbar_wait_warp(&full[s], (item / UNS) & 1))) break;
-                const T gj = gs[j * CW + lane];
-                const T* st = stage + (size_t)s * TR * CW + (size_t)warp * RPW * CW + lane;
-#pragma unroll
-                for (int rr = 0; rr < RPW; ++rr)
-                    if (warp * RPW + rr < rows) wv[rr] -= gj * st[rr * CW];
-                release(&empty[s]);
-            }
-            if (!ok) break;
-            RTy nr = 0;
-            T dl = 0;
-            if (TW && wuni && lane < RPW && warp * RPW + lane < rows)
-                dl = __ldg(wt + row0 + warp * RPW + lane);
-#pragma unroll
-            for (int rr = 0; rr < RPW; ++rr) {
-                const int row = warp * RPW + rr;
-                T d = 0;
-                if (TW) d = __shfl_sync(0xffffffffu, dl, rr);
-                if (row < rows) {
-                    // BF16 storage of the basis (an accuracy trial): the vector
-                    // kept is the rounded one, and beta is its norm
-                    if (sizeof(T) == 4 && r.basis_bf16)
-                        wv[rr] = (T)__bfloat162float(__float2bfloat16_rn((float)wv[rr]));
-                    w[(row0 + row) * CW + lane] = wv[rr];
-                    if (GC) gcopy[(row0 + row) * CW] = wv[rr] * __ldg(gm + row0 + row);
-                    if (TW && !wuni) d = __ldg(wt + row0 + row);
-                    if (TW) nr += (RTy)(wv[rr] * d) * (RTy)wv[rr];
-                    else nr += (RTy)wv[rr] * (RTy)wv[rr];
+                for (int rr = 0; rr < RPW; ++rr) {
+                    const int row = warp * RPW + rr;
+                    wv[rr] = row < rows ? wbuf[(size_t)b * TR * CW + row * CW + lane] : (T)0;
                 }
+                release(&wempty[b]);
+                for (int j = 0; j < i; ++j, ++item) {
+                    const int s = (int)(item % UNS);
+                    if (!(ok = mbar_wait_warp(&full[s], (item / UNS) & 1))) break;
+                    const T gj = gs[j * CW + lane];
+                    const T* st = stage + (size_t)s * TR * CW + (size_t)warp * RPW * CW + lane;
+#pragma unroll
+                    for (int rr = 0; rr < RPW; ++rr)
+                        if (warp * RPW + rr < rows) wv[rr] -= gj * st[rr * CW];
+                    release(&empty[s]);
+                }
+                if (!ok) break;
+                RTy nr = 0;
+                T dl = 0;
+                if (TW && wuni && lane < RPW && warp * RPW + lane < rows)
+                    dl = __ldg(wt + row0 + warp * RPW + lane);
+#pragma unroll
+                for (int rr = 0; rr < RPW; ++rr) {
+                    const int row = warp * RPW + rr;
+                    T d = 0;
+                    if (TW) d = __shfl_sync(0xffffffffu, dl, rr);
+                    if (row < rows) {
+                        // BF16 storage of the basis (an accuracy trial): the vector
+                        // kept is the rounded one, and beta is its norm
+                        if (sizeof(T) == 4 && r.basis_bf16)
+                            wv[rr] = (T)__bfloat162float(__float2bfloat16_rn((float)wv[rr]));
+                        w[(row0 + row) * CW + lane] = wv[rr];
+                        if (GC) gcopy[(row0 + row) * CW] = wv[rr] * __ldg(gm + row0 + row);
+                        if (TW && !wuni) d = __ldg(wt + row0 + row);
+                        if (TW) nr += (RTy)(wv[rr] * d) * (RTy)wv[rr];
+                        else nr += (RTy)wv[rr] * (RTy)wv[rr];
+                    }
+                }
+                acc += (double)nr;
             }
-            acc += (double)nr;
+            // the warps' sums of the segment; a warp that gave up still arrives
+            if (seg > s0) asm volatile("bar.sync 1, %0;" ::"n"(CWARPS * 32) : "memory");
+            red[warp][lane] = acc;
+            asm volatile("bar.sync 1, %0;" ::"n"(CWARPS * 32) : "memory");
+            if (warp == 0) {
+                double sum = 0.0;
+#pragma unroll
+                for (int qq = 0; qq < CWARPS; ++qq) sum += red[qq][lane];
+                part_nrm[((int64_t)blk * r.useg + seg) * CW + lane] = sum;
+            }
         }
     }
     if (!ok) s_fail = 1;
-    red[warp][lane] = acc;
     __syncthreads();
     if (s_fail) {
         if (threadIdx.x == 0) atomicCAS(r.err, DERR_NONE, DERR_TIMEOUT);
         return;
-    }
-    if (warp == 0) {
-        double sum = 0.0;
-#pragma unroll
-        for (int qq = 0; qq < CWARPS; ++qq) sum += red[qq][lane];
-        part_nrm[(int64_t)blk * CW + lane] = sum;
     }
     // The last block of this chunk forms beta_{i+1}, the new scale s_i and the
     // breakdown test for the chunk's columns (no extra launch).
     __shared__ int s_last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&r.cnt_upd[ch], 1) == nblk - 1;
+    if (threadIdx.x == 0) s_last = atomicAdd(&r.cnt_upd[ch], 1) == (int)gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
     {
+        constexpr int F = 8;                     // loads in flight
         double ps = 0.0;
-        for (int b = warp; b < nblk; b += UWARPS)
-            ps += part_nrm[(int64_t)b * CW + lane];
+        for (int b0 = warp; b0 < nnrm; b0 += UWARPS * F) {
+            double v[F];
+#pragma unroll
+            for (int f = 0; f < F; ++f)
+                v[f] = b0 + f * UWARPS < nnrm ? part_nrm[(int64_t)(b0 + f * UWARPS) * CW + lane] : 0.0;
+#pragma unroll
+            for (int f = 0; f < F; ++f) ps += v[f];
+        }
         red[warp][lane] = ps;
     }
     __syncthreads();
@@ -905,10 +917,16 @@ cudaError_t launch_dots_w(const Run& r, int i, cudaStream_t st)
     static std::atomic<uint64_t> attr{0};
     const cudaError_t e = smem_limit_once(attr, reorth_dots_kernel<T, TW>, dots_smem<T>(kMaxSteps));
     if (e != cudaSuccess) return e;
-    // two blocks per SM: where the row blocks do not give them, several blocks
-    // share a row block's vectors
+    // Two blocks per SM: where the row blocks do not give them, several blocks
+    // share a row block's vectors.  FP64, which is bound by the FP64 units, takes
+    // one group per block: the last blocks end together, and a short last group
+    // idles warps of its own block only (200k rows, 80 columns, 40 steps: 89.7 ->
+    // 65.6 ms; FP32 pays the extra w and q tiles: 600k rows, 128 columns: 29.3 ->
+    // 38 ms).  Row blocks of a few tiles would not pay the start of the pipeline
+    // (16k rows: 7.1 -> 7.8 ms; 64k rows: 8.9 -> 8.65 ms).
     const int groups = (i + JB - 1) / JB;
-    const int parts = std::min(groups, std::max(1, 2 * 152 / (r.nblk * r.nchunk)));
+    const int parts = sizeof(T) == 8 && r.n >= (int64_t)1000 * r.nblk
+                          ? groups : std::min(groups, std::max(1, 2 * 152 / (r.nblk * r.nchunk)));
     reorth_dots_kernel<T, TW><<<dim3(r.nblk, r.nchunk, parts), DTHREADS,
                                 dots_smem<T>((groups + parts - 1) / parts * JB), st>>>(r, i);
     return cudaGetLastError();
@@ -941,7 +959,20 @@ cudaError_t launch_update_w(const Run& r, int i, cudaStream_t st)
     const cudaError_t e =
         smem_limit_once(attr, reorth_update_kernel<T, TW, GC>, update_smem<T>(kMaxSteps));
     if (e != cudaSuccess) return e;
-    reorth_update_kernel<T, TW, GC><<<dim3(r.nblk * r.uparts, r.nchunk), UTHREADS, update_smem<T>(i), st>>>(r, i);
+    // Blocks per row block: the divisor of its segments with the least rounds of
+    // resident blocks per row block, and on a tie the fewest blocks (600k rows, 128
+    // columns: 28.3 -> 24.4 ms per 30 steps; FP64, 200k rows, 80 columns: 47.2 ->
+    // 32.3 ms per 40 steps).
+    // (One resident block per SM where a late step's coefficients leave room for no
+    // more: 16k rows, 134 steps, 8.60 -> 8.53 ms.)
+    const size_t smem = update_smem<T>(i);
+    const int slots = 152 * (smem > 112 * 1024 ? 1 : 2), blocks = r.nblk * r.nchunk;
+    int parts = 1;
+    for (int p = 2; p <= r.useg; ++p)
+        if (r.useg % p == 0 && ((int64_t)blocks * p + slots - 1) / slots * parts <
+                                   ((int64_t)blocks * parts + slots - 1) / slots * p)
+            parts = p;
+    reorth_update_kernel<T, TW, GC><<<dim3(r.nblk * parts, r.nchunk), UTHREADS, smem, st>>>(r, i);
     return cudaGetLastError();
 }
 
