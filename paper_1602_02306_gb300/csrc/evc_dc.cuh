@@ -353,8 +353,11 @@ __host__ __device__ inline void dc_pair(double p, double b, double q, double* d,
     double c = 1.0, s = 0.0, t = 0.0;
     if (b != 0.0) {
         const double h = 0.5 * (q - p);
-        // tan of the smaller angle: b / (|h| + sqrt(h^2 + b^2)), h's sign
-        t = b / (fabs(h) + sqrt(h * h + b * b));
+        // tan of the smaller angle: b / (|h| + sqrt(h^2 + b^2)), h's sign; entries
+        // whose squares would vanish (b next to equal p and q) scaled up first
+        const double up = fmax(fabs(h), fabs(b)) < 1e-140 ? 0x1p+600 : 1.0;
+        const double hu = h * up, bu = b * up;
+        t = bu / (fabs(hu) + sqrt(hu * hu + bu * bu));
         if (h < 0.0) t = -t;
         c = dc_rsqrt(1.0 + t * t);
         s = t * c;
