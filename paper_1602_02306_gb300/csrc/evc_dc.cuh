@@ -355,9 +355,13 @@ __host__ __device__ inline void dc_pair(double p, double b, double q, double* d,
         const double h = 0.5 * (q - p);
         // tan of the smaller angle: b / (|h| + sqrt(h^2 + b^2)), h's sign; entries
         // whose squares would vanish (b next to equal p and q) scaled up first
-        const double up = fmax(fabs(h), fabs(b)) < 1e-140 ? 0x1p+600 : 1.0;
-        const double hu = h * up, bu = b * up;
-        t = bu / (fabs(hu) + sqrt(hu * hu + bu * bu));
+        const double sq = fma(b, b, h * h);
+        if (sq < 1e-280) {
+            const double hu = 0x1p+600 * h, bu = 0x1p+600 * b;
+            t = bu / (fabs(hu) + sqrt(hu * hu + bu * bu));
+        } else {
+            t = b / (fabs(h) + sqrt(sq));
+        }
         if (h < 0.0) t = -t;
         c = dc_rsqrt(1.0 + t * t);
         s = t * c;

@@ -33,7 +33,7 @@ def test_vanishing_couplings(k):
         alpha.append(([-3.0, -3.0, 2.0, 5.0] + [1.0] * k)[:k])
         beta.append(([0.0, t, t, 0.5] + [t] * k)[:k + 1])
         alpha.append(([2.0, 2.0, -3.0, -3.0] * k)[:k])
-        beta.append(([0.0, t, 3.0, t] + [t, 2.0] * k)[:k + 1])
+        beta.append(([0.0, t, 3.0, t] + [t, 1.0] * k)[:k + 1])
     a = torch.tensor(alpha, dtype=torch.float64).T.contiguous().cuda()
     b = torch.tensor(beta, dtype=torch.float64).T.contiguous().cuda()
     q = torch.zeros(a.shape[1], dtype=torch.float64, device="cuda")
