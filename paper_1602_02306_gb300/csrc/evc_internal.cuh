@@ -218,6 +218,7 @@ cudaError_t launch_stencil_tma(const StencilOp& op, const StencilPass& p, const 
 bool stencil_pair_eligible(const StencilOp& op, size_t tsize);
 cudaError_t launch_stencil_pair(const StencilOp& op, const Run& r, const StencilPass& first,
                                 const StencilPass& second, cudaStream_t st);
+cudaError_t stencil_pair_selftest(long long cycles, int* err);
 // Arnoldi-type estimator (evc_arnoldi.cu)
 template <typename T>
 cudaError_t launch_row_scale(const Run& r, void* w, int64_t cs, cudaStream_t st);

@@ -2,7 +2,9 @@
 // mbarrier wait can never complete (nothing arrives on the barrier) runs the
 // library's bounded wait with a short limit, gives up, records DERR_TIMEOUT in
 // a device word and returns, so the host sees EVC_ETIMEOUT and the context
-// stays usable.  The streaming kernels report a stalled pipeline the same way.
+// stays usable.  The streaming kernels report a stalled pipeline the same way;
+// the one whose end after a failed wait differs from theirs (the pair kernel: many
+// warps issue the copies) is then run with a copy left out.
 #include "evc_internal.cuh"
 #include "evc_bulk.cuh"
 #include "../../include/evc.h"
@@ -37,17 +39,26 @@ int evc_wait_selftest(double limit_ms, int* status)
         return EVC_ECUDA;
     }
     int* flag = nullptr;
-    if (cudaMalloc(&flag, sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc(&flag, 2 * sizeof(int)) != cudaSuccess) {
         cudaGetLastError();
         return EVC_ENOMEM;
     }
     const long long cycles = (long long)(limit_ms * khz);
-    evc::wait_selftest_kernel<<<1, 64>>>(cycles, flag);
-    cudaError_t e = cudaGetLastError();
-    int h = -1;
-    if (e == cudaSuccess) e = cudaMemcpy(&h, flag, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaError_t e = cudaMemset(flag, 0, 2 * sizeof(int));
+    if (e == cudaSuccess) {
+        evc::wait_selftest_kernel<<<1, 64>>>(cycles, flag);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = evc::stencil_pair_selftest(cycles, flag + 1);
+    int h[2] = {-1, -1};
+    if (e == cudaSuccess) e = cudaMemcpy(h, flag, sizeof h, cudaMemcpyDeviceToHost);
     cudaFree(flag);
-    if (e != cudaSuccess) return EVC_ECUDA;
-    *status = h == evc::DERR_TIMEOUT ? EVC_ETIMEOUT : (h == evc::DERR_NONE ? EVC_OK : EVC_ECUDA);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? EVC_ENOMEM : EVC_ECUDA;
+    }
+    for (int f : h)
+        if (f != evc::DERR_TIMEOUT && f != evc::DERR_NONE) return *status = EVC_ECUDA, EVC_OK;
+    *status = h[0] == evc::DERR_TIMEOUT && h[1] == evc::DERR_TIMEOUT ? EVC_ETIMEOUT : EVC_OK;
     return EVC_OK;
 }

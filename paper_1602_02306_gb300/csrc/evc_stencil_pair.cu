@@ -34,7 +34,8 @@
 // (the others wait for it: 1000).
 //
 // Every wait is bounded and records DERR_TIMEOUT; a warp that gave up still takes
-// part in every barrier of the plane loop.
+// part in every barrier of the plane loop, and the block waits for the copies it
+// issued before it exits.
 #include "evc_internal.cuh"
 #include "evc_bulk.cuh"
 
@@ -43,6 +44,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -109,7 +111,7 @@ struct Geo {
     static constexpr int X0 = 2 * PSTEP, Y0 = X0 + 2 * XSTEP, C0 = Y0 + 4 * YSTEP;
     static constexpr int PTS = C0 + 4 * CSTEP;
     static constexpr int BOXES = 2 + 2 + 4 + 4;
-    static constexpr uint32_t TX_BYTES = (TS * TS + 4 * TS + 4 * TS + 4) * NC * 4;
+    static_assert(BOXES <= NCW, "a warp issues at most one box of a plane");
     // one plane of u by parity [TS + 2][2][PP]; a patch on the rim also reads one
     // row or point before or after it, for u values that nobody uses: the memory
     // there is the ring's, another plane's or the pad's
@@ -133,6 +135,8 @@ struct PairArgs {
     int64_t out_cs;
     const int* chunk_active;
     int* err;
+    long long limit;         // clock cycles that a wait may take
+    int have;                // planes whose first box is issued: all but in the self-test
 };
 
 // Maps over [chunk][y + N z][x / 2][x % 2][CW], by box (NC columns each): a
@@ -153,13 +157,13 @@ __device__ __forceinline__ void load5(uint32_t dst, const CUtensorMap* map, int 
 }
 
 // Bounded wait that also gives up once the block's failure flag is set.
-__device__ __forceinline__ bool wait_or(uint64_t* bar, uint32_t parity, volatile int* fail)
+__device__ __forceinline__ bool wait_or(uint64_t* bar, uint32_t parity, volatile int* fail, long long limit)
 {
     if (mbar_test(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_test(bar, parity)) {
         if (*fail) return false;
-        if (clock64() - t0 > kWaitCycles) {
+        if (clock64() - t0 > limit) {
             *fail = 1;
             return false;
         }
@@ -184,10 +188,10 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
     const uint32_t xbase = smem_addr(raw), ubase = xbase + LA * G::XB;
     __shared__ uint64_t full[LA];            // a plane of x has landed
     __shared__ uint64_t udone[2];            // every warp has stored its u of a plane (and read x for it)
-    __shared__ int s_fail;
+    __shared__ int s_fail, s_last[G::BOXES];
     __shared__ int4 boxes[G::BOXES];
     if (threadIdx.x == 0) {
-        for (int s = 0; s < LA; ++s) mbar_init(&full[s], 1);
+        for (int s = 0; s < LA; ++s) mbar_init(&full[s], G::BOXES);
         for (int s = 0; s < 2; ++s) mbar_init(&udone[s], NCW);
         s_fail = 0;
         mbar_init_fence();
@@ -206,7 +210,9 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
 
     // The boxes of a plane: {map, x, y, position in the stage}.  The two rows or
     // columns of an arm are even-aligned (N, x0 and y0 are even), so they wrap
-    // together.  Box b of plane t (z0 - 2 + t) is issued by warp b % NCW.
+    // together.  Box b of plane t (z0 - 2 + t) is issued by warp b, which alone
+    // announces its bytes: a plane that some warps no longer issue, because a wait
+    // gave up meanwhile, can still be waited for (below).
     if (threadIdx.x < G::BOXES) {
         const int b = threadIdx.x;
         int4 e;
@@ -217,19 +223,17 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
         boxes[b] = e;
     }
     __syncthreads();
+    const int pts = warp < 2 ? TS * G::H : warp < 4 ? 2 * TS : warp < 8 ? 2 * G::H : 1;    // of this warp's box
+    int last = -1;                           // last plane that this warp issued its box of
     auto issue = [&](int t, int stage) {
-        if (t >= nplane || l32 != 0 || *fail) return;
+        if (warp >= G::BOXES || t >= nplane || l32 != 0 || *fail || (t >= a.have && warp == 0)) return;
         uint64_t* bar = &full[stage];
-        if (warp == 0) mbar_arrive_expect_tx(bar, G::TX_BYTES);
         int z = z0 - 2 + t;
         z = z < 0 ? z + N : z >= N ? z - N : z;
-#pragma unroll
-        for (int b = 0; b < (G::BOXES + NCW - 1) / NCW; ++b) {
-            if (b * NCW + warp >= G::BOXES) break;
-            const int4 e = boxes[b * NCW + warp];
-            load5(xbase + stage * G::XB + e.w * NC * 4, &maps.box[e.x], grp * NC, e.y & 1, e.y >> 1, z * N + e.z,
-                  ch, bar);
-        }
+        const int4 e = boxes[warp];
+        mbar_arrive_expect_tx(bar, pts * NC * 4);
+        load5(xbase + stage * G::XB + e.w * NC * 4, &maps.box[e.x], grp * NC, e.y & 1, e.y >> 1, z * N + e.z, ch, bar);
+        last = t;
     };
 #pragma unroll
     for (int t = 0; t < LA; ++t) issue(t, t);
@@ -291,7 +295,7 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
         F2 xw[3][4], uw[3][4];
         bool ok = true;
         auto take = [&](int stage, uint32_t parity, F2* x) {        // own points of a plane
-            ok = ok && __all_sync(0xffffffffu, wait_or(&full[stage], parity, fail));
+            ok = ok && __all_sync(0xffffffffu, wait_or(&full[stage], parity, fail, a.limit));
 #pragma unroll
             for (int q = 0; q < 4; ++q) x[q] = lds(own[q], stage * G::XB);
         };
@@ -324,7 +328,7 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
             if (j >= 1) {
                 // every warp is done with plane j - 1 of u, hence with plane j of x,
                 // whose stage takes the next plane to load
-                ok = ok && __all_sync(0xffffffffu, wait_or(&udone[(s + 1) & 1], ((j - 1) >> 1) & 1, fail));
+                ok = ok && __all_sync(0xffffffffu, wait_or(&udone[(s + 1) & 1], ((j - 1) >> 1) & 1, fail, a.limit));
                 if (j == 1) issue(LA, 0);
                 issue(j + LA, s % LA);
             }
@@ -366,11 +370,24 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
         }
     }
     __syncthreads();
-    // Every plane issued was waited for, unless a wait gave up: then the copies
-    // still in flight get a millisecond before the shared memory is released.
-    if (threadIdx.x == 0 && *fail) {
-        atomicCAS(a.err, DERR_NONE, DERR_TIMEOUT);
-        for (const long long t0 = clock64(); clock64() - t0 < 2000000;) {}
+    // Every plane issued was waited for, unless a wait gave up.  Then, before the
+    // shared memory is released: arrive in the place of the warps that issued no box
+    // of a plane any more, and wait (again with the limit) for the others' boxes.  A
+    // plane was issued only once every warp had seen the one before it in its stage,
+    // so the last LA planes are the ones that can be in flight.
+    if (*fail) {
+        if (l32 == 0 && warp < G::BOXES) s_last[warp] = last;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            atomicCAS(a.err, DERR_NONE, DERR_TIMEOUT);
+            int most = -1;
+            for (int b = 0; b < G::BOXES; ++b) most = max(most, s_last[b]);
+            for (int t = max(0, most - LA + 1); t <= most; ++t) {
+                for (int b = 0; b < G::BOXES; ++b)
+                    if (s_last[b] < t) mbar_arrive(&full[t % LA]);
+                mbar_wait_for(&full[t % LA], (t / LA) & 1, a.limit);
+            }
+        }
     }
     __syncthreads();
 }
@@ -501,11 +518,47 @@ cudaError_t launch_stencil_pair(const StencilOp& op, const Run& r, const Stencil
     a.out_cs = second.out_cs;
     a.chunk_active = r.chunk_active + c0;
     a.err = r.err;
+    a.limit = kWaitCycles;
+    a.have = INT_MAX;
     const Shape sh = choose_shape(op.N, r.nchunk, op.zb > 0 ? op.zb : 64);
     a.zb = sh.zb;
     return sh.ts == 16   ? launch_ts<16>(op, p, a, cn, st)
            : sh.ts == 14 ? launch_ts<14>(op, p, a, cn, st)
                          : launch_ts<12>(op, p, a, cn, st);
+}
+
+// The failure path on a 12^3 grid: plane 2 lacks its first box, so the waits for it
+// give up after `cycles` and the block winds down with the plane's other boxes in
+// flight.  *err (device memory) receives DERR_TIMEOUT.
+cudaError_t stencil_pair_selftest(long long cycles, int* err)
+{
+    constexpr int N = 12;
+    const size_t vec = (size_t)N * N * N * CW;
+    float* buf = nullptr;                        // x, out, then a chunk's flag
+    cudaError_t e = cudaMalloc(&buf, (2 * vec + 1) * sizeof(float));
+    if (e != cudaSuccess) return e;
+    PairArgs a{};
+    a.N = N;
+    a.zb = N;
+    a.out = buf + vec;
+    a.out_cs = (int64_t)vec;
+    int* active = reinterpret_cast<int*>(buf + 2 * vec);
+    a.chunk_active = active;
+    a.err = err;
+    a.limit = cycles;
+    a.have = 2;
+    StencilOp op{};
+    op.N = N;
+    StencilPass p{};
+    p.in = buf;
+    p.in_cs = (int64_t)vec;
+    const int one = 1;
+    e = cudaMemset(buf, 0, 2 * vec * sizeof(float));
+    if (e == cudaSuccess) e = cudaMemcpy(active, &one, sizeof one, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = launch_ts<12>(op, p, a, 1, nullptr);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    cudaFree(buf);
+    return e;
 }
 
 }  // namespace evc
