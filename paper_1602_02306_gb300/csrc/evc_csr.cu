@@ -224,7 +224,11 @@ csr_pass_kernel(CArgs a)
 // 36 warps per SM: the registers that this leaves (56) hold the batch, and the
 // time no longer depends on the block size (two gathers in flight: 30 % slower;
 // eight without the bound: 1.18, 1.51 and 1.73 ms with 128, 64 and 256 threads).
-// (Past a row's end: its own row of x, times zero.)  ms per pass, before | now:
+// FP32 rows are padded to whole batches (their own row of x, times zero): smaller
+// batches for the rest cost more than the gathers they save (2M rows, six passes:
+// 25.5 | 26.2 to 27.0 ms).  FP64 rows are not: a padded entry takes the FP64 units,
+// which bound the pass, as long as a real one (500k rows of 3, 5, 7 and 13 entries,
+// six passes: 3.7, 3.7, 3.7, 6.5 | 2.4, 2.9, 3.4, 5.4 ms).  ms per pass, before | now:
 //   64 columns x 2 shifts, power-law rows (mean 29), FP32, T^-1 process: 600k
 //   rows 1.44 | 1.00, 2M 4.85 | 4.41; Jacobi: 2M 5.28 | 4.60 and 0.16 more in the
 //   kernel that writes the copy, 600k 1.66 | 1.10, 30k (one row of 2000 entries
@@ -278,19 +282,34 @@ csr_gather_kernel(CArgs a)
             nval = ld_once(val + k0 + LPR + sub, once);
         }
         const int cnt = (int)min((int64_t)LPR, mx - k0);
+        auto batch = [&](auto size, int t) {
+            constexpr int B = decltype(size)::value;
+            Pack<T> xv[B];
 #pragma unroll
-        for (int t = 0; t < LPR; t += U) {
-            if (t >= cnt) break;
-            Pack<T> xv[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u)
+            for (int u = 0; u < B; ++u)
                 xv[u] = ldg16(y + (int64_t)__shfl_sync(0xffffffffu, mycol, grp * LPR + t + u) * CW);
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
+            for (int u = 0; u < B; ++u) {
                 const T v = __shfl_sync(0xffffffffu, myval, grp * LPR + t + u);
 #pragma unroll
                 for (int w = 0; w < W; ++w) acc[w] = fma_rn(v, xv[u].v[w], acc[w]);
             }
+        };
+        if constexpr (sizeof(T) == 4) {
+            static_assert(sizeof(T) == 8 || U == LPR, "one batch holds a row's lanes");
+            batch(std::integral_constant<int, U>(), 0);
+        } else {
+            int t = 0;
+            for (; t + U <= cnt; t += U) batch(std::integral_constant<int, U>(), t);
+            if (cnt & 4) {
+                batch(std::integral_constant<int, 4>(), t);
+                t += 4;
+            }
+            if (cnt & 2) {
+                batch(std::integral_constant<int, 2>(), t);
+                t += 2;
+            }
+            if (cnt & 1) batch(std::integral_constant<int, 1>(), t);
         }
     }
     if (!valid) return;
