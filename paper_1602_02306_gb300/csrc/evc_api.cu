@@ -179,6 +179,22 @@ int choose_useg(int64_t n, int nblk)
     return n >= (int64_t)2048 * nblk && 2 * reorth_max_blocks(n) >= 3 * nblk ? 3 : 2;
 }
 
+// Whether a CSR run under Jacobi gathers from a copy of q_i scaled by m (see Run::gcopy;
+// the bits are the same either way).  The copy costs a written and, for the diagonal, a
+// read vector per step and saves a product and a gathered m per entry and, where the 32
+// columns of a chunk have several shifts, per column: it pays for long rows.  FP64 is
+// bound by its products: always.  Passes and updates of eight steps, ms, without | with
+// the copy: 300k rows, 64 columns, FP32, 5, 9, 13 and 27 random entries per row 1.86 |
+// 2.08, 2.08 | 2.23, 2.31 | 2.38, 3.04 | 2.88; 40 columns of two shifts, 3, 5 and 7 entries
+// 2.94 | 2.90, 3.23 | 3.03, 3.55 | 3.16; FP64, 64 columns, 3 and 13 entries 4.90 | 4.70,
+// 10.2 | 7.28.  (A band of neighbouring entries, whose m are in L1, gains less.)
+bool copy_pays(const evc_ctx* c, int S, int m)
+{
+    if (c->precision == EVC_FP64) return true;
+    const bool one_shift = S == 1 || m % CW == 0;
+    return c->nnz >= (one_shift ? 16 : 5) * c->n;
+}
+
 struct Layout {
     size_t total;
     int nchunk, ncol, nblk;
@@ -287,7 +303,7 @@ size_t carve(const evc_ctx* c, int S, int m, int kmax, char* base, Run& r, void*
     r.basis_bf16 = c->basis_bf16;
     r.arnoldi = c->method == EVC_METHOD_ARNOLDI ? 1 : 0;
     r.hess = r.arnoldi ? D((size_t)kmax * (kmax + 1) / 2 * ncol) : nullptr;
-    r.gcopy = c->op == OP_CSR && uses_jac(c) && !r.tinv && !r.arnoldi;
+    r.gcopy = c->op == OP_CSR && uses_jac(c) && !r.tinv && !r.arnoldi && copy_pays(c, S, m);
     return off;
 }
 
