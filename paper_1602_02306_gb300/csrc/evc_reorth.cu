@@ -911,22 +911,54 @@ size_t update_smem(int i)
            (2 * UNS + 4) * sizeof(uint64_t);
 }
 
+// Blocks that share a row block's vectors at step i, by the row blocks of all chunks.
+// Two blocks per SM: where the row blocks do not give them, several blocks share.
+// FP64, which is bound by the FP64 units, takes one group per block: the last blocks
+// end together, and a short last group idles warps of its own block only (200k rows,
+// 80 columns, 40 steps: 89.7 -> 65.6 ms; FP32 pays the extra w and q tiles: 600k rows,
+// 128 columns: 29.3 -> 38 ms).  Not where the row blocks alone fill their last round,
+// of two blocks per SM or, below one round, of one (262k rows, 128 columns, steps 9 to
+// 24: 31.9 | 33.1 ms; 64 columns: 17.2 | 19.8).  Row blocks of a few tiles would not pay
+// the start of the pipeline (16k rows: 7.1 -> 7.8 ms; 64k rows: 8.9 -> 8.65 ms).
+// FP64 with T^-1: the weighting of the w and q tiles costs a block as much as four
+// vectors, and a block cannot be faster than that of eight: the fewest rounds at that
+// price, a round of at most one block per SM taking 0.6 of one of two, and sharing
+// only where it gains 5 % (steps 17 to 24, ms, one block | one per group | this: 1M
+// rows, 64 columns 41.7 | 54.7 | 41.7; 200k rows, 32, 64 and 96 columns 10.8, 10.8, 19.0 |
+// 7.8, 14.4, 18.2 | 7.2, 10.7, 18.6).
+int dots_parts(int i, int blocks, bool long_blocks, bool fp64, bool tw)
+{
+    const int groups = (i + JB - 1) / JB, slots = 2 * 152;
+    const int rounds = (blocks + slots - 1) / slots;
+    if (!fp64 || (!long_blocks && !tw)) return std::min(groups, std::max(1, slots / blocks));
+    if (!tw) {
+        const bool full = blocks >= 0.95 * slots * rounds || (blocks > 128 && blocks <= slots / 2 && groups <= 3);
+        return full ? 1 : groups;
+    }
+    int best = 1;
+    double least = 0.0;
+    for (int p = 1; p <= groups; ++p) {
+        int work = 0;
+        for (int q = 0; q < p; ++q) work += std::max(dots_count(i, q, p), 8) + 4;
+        const int64_t b = (int64_t)blocks * p;
+        const double cost = (b <= slots / 2 ? 0.6 : (double)((b + slots - 1) / slots)) * work / p;
+        if (p == 1) least = 0.95 * cost;
+        else if (cost < least) {
+            least = cost;
+            best = p;
+        }
+    }
+    return best;
+}
+
 template <typename T, bool TW>
 cudaError_t launch_dots_w(const Run& r, int i, cudaStream_t st)
 {
     static std::atomic<uint64_t> attr{0};
     const cudaError_t e = smem_limit_once(attr, reorth_dots_kernel<T, TW>, dots_smem<T>(kMaxSteps));
     if (e != cudaSuccess) return e;
-    // Two blocks per SM: where the row blocks do not give them, several blocks
-    // share a row block's vectors.  FP64, which is bound by the FP64 units, takes
-    // one group per block: the last blocks end together, and a short last group
-    // idles warps of its own block only (200k rows, 80 columns, 40 steps: 89.7 ->
-    // 65.6 ms; FP32 pays the extra w and q tiles: 600k rows, 128 columns: 29.3 ->
-    // 38 ms).  Row blocks of a few tiles would not pay the start of the pipeline
-    // (16k rows: 7.1 -> 7.8 ms; 64k rows: 8.9 -> 8.65 ms).
     const int groups = (i + JB - 1) / JB;
-    const int parts = sizeof(T) == 8 && r.n >= (int64_t)1000 * r.nblk
-                          ? groups : std::min(groups, std::max(1, 2 * 152 / (r.nblk * r.nchunk)));
+    const int parts = dots_parts(i, r.nblk * r.nchunk, r.n >= (int64_t)1000 * r.nblk, sizeof(T) == 8, TW);
     reorth_dots_kernel<T, TW><<<dim3(r.nblk, r.nchunk, parts), DTHREADS,
                                 dots_smem<T>((groups + parts - 1) / parts * JB), st>>>(r, i);
     return cudaGetLastError();
