@@ -434,7 +434,9 @@ __device__ __forceinline__ int64_t tri(int a, int b)
 // alpha_i = h_{i-1}.  One block of RW warps per (chunk, j): warp q sums the row
 // blocks b = q, q+RW, ... for the 32 columns (one coalesced 256-byte load per
 // b), then the warps' sums are added in warp order (fixed summation order).
+// F of a warp's row blocks are in flight at a time: sixteen are all of 64 row blocks.
 constexpr int RW = 4;
+template <int F>
 __global__ void __launch_bounds__(RW * 32)
 reorth_reduce_kernel(Run r, int i)
 {
@@ -443,8 +445,6 @@ reorth_reduce_kernel(Run r, int i)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ double sh[RW][CW], sg[RW][CW];
     double ah = 0.0, ag = 0.0;
-    // sixteen row blocks at a time in flight: all of a small problem's
-    constexpr int F = 16;
     for (int b0 = warp; b0 < r.nblk; b0 += RW * F) {
         double vh[F], vg[F];
 #pragma unroll
@@ -972,7 +972,12 @@ cudaError_t launch_dots(const Run& r, int i, cudaStream_t st)
 
 cudaError_t launch_reduce(const Run& r, int i, cudaStream_t st)
 {
-    reorth_reduce_kernel<<<r.nchunk * i, RW * 32, 0, st>>>(r, i);
+    // no more in flight than a warp has: with many columns the loads left out count
+    // (3 row blocks, 16384 columns, step 64: sixteen 392 us, four 227 with coef)
+    const dim3 grid(r.nchunk * i);
+    if (r.nblk <= RW) reorth_reduce_kernel<1><<<grid, RW * 32, 0, st>>>(r, i);
+    else if (r.nblk <= 4 * RW) reorth_reduce_kernel<4><<<grid, RW * 32, 0, st>>>(r, i);
+    else reorth_reduce_kernel<16><<<grid, RW * 32, 0, st>>>(r, i);
     return cudaGetLastError();
 }
 
