@@ -195,6 +195,10 @@ inline int reorth_max_blocks(int64_t n)
     return (int)(m < 65535 ? (m > 0 ? m : 1) : 65535);
 }
 
+// Bytes of a tile of the update kernel, and its rows by the size of an element.
+constexpr int kUpdateStage = 8192;
+constexpr int update_rows(int tsize) { return kUpdateStage / (CW * tsize); }
+
 // Kernel launchers (T = float for EVC_MIXED, double for EVC_FP64).
 // Diagonal preconditioning of an operator pass: none, M (A - sigma I) M with
 // the Jacobi M, or T (A - sigma I) with T = M^2 (T^{-1}-inner-product mode).

@@ -200,7 +200,7 @@ constexpr int NPROD = 2;                        // producer warps, dot kernel
 constexpr int DTHREADS = (CWARPS + NPROD) * 32; // threads of the dot kernel
 static_assert(CWARPS % NPROD == 0, "a consumer warp's ring must have one producer");
 constexpr int DNS = CWARPS * NSW;               // stages, dot kernel
-constexpr int USTAGE = 8192;                    // bytes per stage, update kernel
+constexpr int USTAGE = kUpdateStage;            // bytes per stage, update kernel
 constexpr int UNS = 10;                         // stages, update kernel
 constexpr int UWARPS = CWARPS + NPROD;          // warps of the update kernel
 constexpr int UTHREADS = UWARPS * 32;           // threads of the update kernel
@@ -997,18 +997,27 @@ cudaError_t launch_update_w(const Run& r, int i, cudaStream_t st)
         smem_limit_once(attr, reorth_update_kernel<T, TW, GC>, update_smem<T>(kMaxSteps));
     if (e != cudaSuccess) return e;
     // Blocks per row block: the divisor of its segments with the least rounds of
-    // resident blocks per row block, and on a tie the fewest blocks (600k rows, 128
-    // columns: 28.3 -> 24.4 ms per 30 steps; FP64, 200k rows, 80 columns: 47.2 ->
-    // 32.3 ms per 40 steps).
+    // resident blocks times a block's tiles, and on a tie the fewest blocks (600k rows,
+    // 128 columns: 28.3 -> 24.4 ms per 30 steps; FP64, 200k rows, 80 columns: 47.2 ->
+    // 32.3 ms per 40 steps).  A block's start counts as half a tile (1024 rows, 8192
+    // columns, FP32, 30 steps: one block 4.2, two 5.2 ms).  Below one block per SM a block
+    // has the SM to itself and takes some 0.65 of the time (FP64 and T^-1 0.7, and 0.6
+    // where it fills all SMs; 262k rows, 64 columns, FP64: one block 18.5, three 19.5 ms;
+    // 200k rows: 16.9, 14.8).
     // (One resident block per SM where a late step's coefficients leave room for no
     // more: 16k rows, 134 steps, 8.60 -> 8.53 ms.)
     const size_t smem = update_smem<T>(i);
-    const int slots = 152 * (smem > 112 * 1024 ? 1 : 2), blocks = r.nblk * r.nchunk;
+    const int per_sm = smem > 112 * 1024 ? 1 : 2, slots = 152 * per_sm, blocks = r.nblk * r.nchunk;
+    const int64_t tiles = ((r.n + r.nblk - 1) / r.nblk + update_rows(sizeof(T)) - 1) / update_rows(sizeof(T));
+    const double alone = sizeof(T) == 4 && !TW ? 0.65 : blocks > 144 ? 0.6 : 0.7;
+    auto cost = [&](int p) {
+        const int64_t b = (int64_t)blocks * p;
+        const double rounds = per_sm == 2 && b <= 152 ? alone : (double)((b + slots - 1) / slots);
+        return rounds * ((double)((tiles + p - 1) / p) + 0.5);
+    };
     int parts = 1;
     for (int p = 2; p <= r.useg; ++p)
-        if (r.useg % p == 0 && ((int64_t)blocks * p + slots - 1) / slots * parts <
-                                   ((int64_t)blocks * parts + slots - 1) / slots * p)
-            parts = p;
+        if (r.useg % p == 0 && cost(p) < cost(parts)) parts = p;
     reorth_update_kernel<T, TW, GC><<<dim3(r.nblk * parts, r.nchunk), UTHREADS, smem, st>>>(r, i);
     return cudaGetLastError();
 }
