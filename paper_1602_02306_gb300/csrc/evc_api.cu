@@ -763,7 +763,7 @@ int enqueue_cheb_factored(evc_ctx* ctx, const Run& r, int step, const void* x, i
         const double sg = last ? ctx->cheb_sign : 1.0;
         // one kernel for both passes of a pair where there is one: it reads its
         // operand with a halo, so it never writes in place
-        const bool fused = F.pair && stencil_pair_eligible(ctx->sten, sizeof(T));
+        const bool fused = F.pair && stencil_pair_eligible(ctx->sten, sizeof(T), r.nchunk);
         void* dst = last ? out : fused && cur == Wb ? Wa : Wb;
         const int64_t dst_cs = last ? out_cs : wcs;
         StencilPass p{}, pa{};

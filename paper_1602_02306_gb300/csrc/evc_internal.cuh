@@ -219,7 +219,7 @@ cudaError_t launch_stencil_tma(const StencilOp& op, const StencilPass& p, const 
                                int64_t n, int* err, int cn, int pmode, cudaStream_t st);
 // The two passes of a conjugate pair of roots of M = p_d(K) in one kernel
 // (evc_stencil_pair.cu): first x -> u, second u -> out; u is not stored.
-bool stencil_pair_eligible(const StencilOp& op, size_t tsize);
+bool stencil_pair_eligible(const StencilOp& op, size_t tsize, int nchunk);
 cudaError_t launch_stencil_pair(const StencilOp& op, const Run& r, const StencilPass& first,
                                 const StencilPass& second, cudaStream_t st);
 cudaError_t stencil_pair_selftest(long long cycles, int* err);

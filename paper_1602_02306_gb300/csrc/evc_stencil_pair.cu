@@ -475,9 +475,19 @@ cudaError_t launch_ts(const StencilOp& op, const StencilPass& p, const PairArgs&
 
 }  // namespace
 
-bool stencil_pair_eligible(const StencilOp& op, size_t tsize)
+// FP32 7-point passes on grids with N even and at least the smallest tile.  Not for
+// many columns on grids of little more than a tile, which the tiles cover one and a
+// half to two times, where the single passes run on patches that march whole lines or
+// overlap in chunk groups.  ms of 6 steps, 2 x 2 patches, pair | single passes: 32
+// chunks, 4 groups, 16 z planes per block N = 18 2.74 | 2.50, 20 2.98 | 2.72, 22 3.38 |
+// 3.15; 64 chunks, one group N = 18 5.40 | 4.67, 20 6.01 | 5.36, 22 6.89 | 6.25.  At N = 24
+// (two tiles, exactly) with 32 chunks it is 3.51 | 4.23, and from N = 26 on, or with less
+// work than this, the pair is faster too (N = 22, 16 chunks, 4 steps 0.88 | 0.93).
+bool stencil_pair_eligible(const StencilOp& op, size_t tsize, int nchunk)
 {
-    return tsize == 4 && op.order == 2 && op.N >= 12 && op.N % 2 == 0 && encode_fn() != nullptr;
+    if (tsize != 4 || op.order != 2 || op.N < 12 || op.N % 2 || encode_fn() == nullptr) return false;
+    const bool patches = op.patch >= 2 && (op.cn > 0 || (op.zb > 0 ? op.zb : 32) >= op.N);
+    return !(patches && op.N > 16 && op.N < 24 && (int64_t)op.N * op.N * op.N * nchunk >= 180000);
 }
 
 // first: x -> u (in, insc, k1, k0); second: u -> out (k1, k0, x, xs, a0, pp, ppc, out).
@@ -485,7 +495,7 @@ cudaError_t launch_stencil_pair(const StencilOp& op, const Run& r, const Stencil
                                 const StencilPass& second, cudaStream_t st)
 {
     const int c0 = op.cn > 0 ? op.c0 : 0, cn = op.cn > 0 ? op.cn : r.nchunk;
-    if (c0 < 0 || c0 + cn > r.nchunk || !stencil_pair_eligible(op, 4)) return cudaErrorInvalidValue;
+    if (c0 < 0 || c0 + cn > r.nchunk || !stencil_pair_eligible(op, 4, r.nchunk)) return cudaErrorInvalidValue;
     if (first.in != second.x || first.in_cs != second.x_cs || first.in == second.out || first.useV ||
         second.useV || second.prev || first.pp || first.x)
         return cudaErrorInvalidValue;
