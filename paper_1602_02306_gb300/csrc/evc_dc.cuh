@@ -45,19 +45,52 @@ namespace evc {
 constexpr double kDcEps = 2.220446049250313e-16;
 
 // The lanes that work on one root: `P` consecutive lanes of a warp, of which
-// this is lane `sub`.  sum() gives every lane the same bits.
+// this is lane `sub`.  sum() gives every lane the same bits.  A lane may do the
+// work of WAY lanes instead: it keeps their partial sums apart and adds them in the
+// order of the shuffles, so that the bits are those of WAY P lanes.
 struct DcLanes {
     int sub, P;
     unsigned mask;
-    template <typename R>
-    __host__ __device__ R sum(R v) const
+    template <typename R, int WAY>
+    __host__ __device__ R sum(R (&v)[WAY]) const
     {
+#pragma unroll
+        for (int o = WAY >> 1; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < o; ++q) v[q] += v[q + o];
+        R r = v[0];
 #ifdef __CUDA_ARCH__
-        for (int o = P >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+        for (int o = P >> 1; o > 0; o >>= 1) r += __shfl_xor_sync(mask, r, o);
 #endif
-        return v;
+        return r;
+    }
+    template <typename R, int WAY>
+    __host__ __device__ R product(R (&v)[WAY]) const
+    {
+#pragma unroll
+        for (int o = WAY >> 1; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < o; ++q) v[q] *= v[q + o];
+        R r = v[0];
+#ifdef __CUDA_ARCH__
+        for (int o = P >> 1; o > 0; o >>= 1) r *= __shfl_xor_sync(mask, r, o);
+#endif
+        return r;
     }
 };
+
+// term(j, q) for this lane's j < K: j = sub + q P, q < WAY, and again WAY P further on.
+template <int WAY, typename F>
+__host__ __device__ inline void dc_each(int K, const DcLanes& g, F&& term)
+{
+    int j = g.sub;
+    for (; j + (WAY - 1) * g.P < K; j += WAY * g.P)
+#pragma unroll
+        for (int q = 0; q < WAY; ++q) term(j + q * g.P, q);
+#pragma unroll
+    for (int q = 0; q < WAY - 1; ++q)
+        if (j + q * g.P < K) term(j + q * g.P, q);
+}
 
 // 1/x to working precision: the hardware's approximation (20 bits) and two
 // Newton steps.  x is a difference of distinct poles or of a pole and a root.
@@ -78,6 +111,16 @@ __host__ __device__ inline float dc_rcp(float x)
     return __fdividef(1.0f, x);
 #else
     return 1.0f / x;
+#endif
+}
+// A product that no compiler fuses with a sum (all sums of products here are fused,
+// or not, in so many words: the variants of the solver have to agree bit by bit).
+__host__ __device__ inline float dc_mul(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
 #endif
 }
 __host__ __device__ inline double dc_rsqrt(double x)
@@ -104,15 +147,15 @@ struct DcSums {
 __host__ __device__ inline float dc_step(float ai, float aj, float A, float B, float f, bool last)
 {
     const float c = f - A - B;
-    const float a = ai * (f - B) + aj * (f - A);
+    const float a = fmaf(aj, f - A, ai * (f - B));
     const float b = ai * aj * f;
-    const float disc = a * a - 4.0f * b * c;
+    const float disc = fmaf(a, a, -(4.0f * b * c));
     const float q = sqrtf(disc > 0.0f ? disc : 0.0f);
     float eta;
     if (last) eta = a >= 0.0f ? (a + q) / (2.0f * c) : 2.0f * b / (a - q);
     else eta = a <= 0.0f ? (a - q) / (2.0f * c) : 2.0f * b / (a + q);
     // f increases: the step must go against its sign (else Newton's step)
-    if (!(f * eta < 0.0f)) eta = -f * ai * aj / (A * aj + B * ai);
+    if (!(f * eta < 0.0f)) eta = -f * ai * aj / fmaf(A, aj, B * ai);
     return eta;
 }
 
@@ -124,47 +167,54 @@ struct DcPoles {
     int K;
 };
 
+template <int WAY>
 __host__ __device__ inline DcSums<double> dc_sums(const DcPoles& p, int split, double org, double mu,
                                                   const DcLanes& g)
 {
-    DcSums<double> s{0, 0, 0, 0};
-    for (int j = g.sub; j < p.K; j += g.P) {
+    // (the left sums are put aside at the first pole of a partial sum to the right: two
+    // FP64 operations per term, not four)
+    double psi[WAY] = {}, phi[WAY] = {}, dpsi[WAY] = {}, dphi[WAY] = {};
+    dc_each<WAY>(p.K, g, [&](int j, int q) {
         const double zj = p.z[j];
         const double t = zj * dc_rcp((p.d[j] - org) - mu);
-        const double l = j <= split ? t : 0.0, r = j <= split ? 0.0 : t;
-        s.psi += l * zj;
-        s.phi += r * zj;
-        s.dpsi += l * l;
-        s.dphi += r * r;
+        if (j > split && j - WAY * g.P <= split) {
+            psi[q] = phi[q];
+            dpsi[q] = dphi[q];
+            phi[q] = dphi[q] = 0.0;
+        }
+        phi[q] = fma(t, zj, phi[q]);
+        dphi[q] = fma(t, t, dphi[q]);
+    });
+#pragma unroll
+    for (int q = 0; q < WAY; ++q) {
+        const int first = g.sub + q * g.P;               // no pole of this sum to the right:
+        if (first + (p.K - 1 - first) / (WAY * g.P) * (WAY * g.P) <= split) {
+            psi[q] = phi[q];
+            dpsi[q] = dphi[q];
+            phi[q] = dphi[q] = 0.0;
+        }
     }
-    s.psi = g.sum(s.psi);
-    s.phi = g.sum(s.phi);
-    s.dpsi = g.sum(s.dpsi);
-    s.dphi = g.sum(s.dphi);
-    return s;
+    return DcSums<double>{g.sum(psi), g.sum(phi), g.sum(dpsi), g.sum(dphi)};
 }
 
+template <int WAY>
 __host__ __device__ inline DcSums<float> dc_sums(const DcPoles& p, int split, int o, float mu,
                                                  const DcLanes& g)
 {
     const float hi = p.hi[o], lo = p.lo[o];
-    DcSums<float> s{0, 0, 0, 0};
-    for (int j = g.sub; j < p.K; j += g.P) {
+    float psi[WAY] = {}, phi[WAY] = {}, dpsi[WAY] = {}, dphi[WAY] = {};
+    dc_each<WAY>(p.K, g, [&](int j, int q) {
         const float r = dc_rcp(((p.hi[j] - hi) + (p.lo[j] - lo)) - mu);
-        const float v = p.z2[j] * r, t = v * r;
+        const float v = dc_mul(p.z2[j], r), t = dc_mul(v, r);
         if (j <= split) {
-            s.psi += v;
-            s.dpsi += t;
+            psi[q] += v;
+            dpsi[q] += t;
         } else {
-            s.phi += v;
-            s.dphi += t;
+            phi[q] += v;
+            dphi[q] += t;
         }
-    }
-    s.psi = g.sum(s.psi);
-    s.phi = g.sum(s.phi);
-    s.dpsi = g.sum(s.dpsi);
-    s.dphi = g.sum(s.dphi);
-    return s;
+    });
+    return DcSums<float>{g.sum(psi), g.sum(phi), g.sum(dpsi), g.sum(dphi)};
 }
 
 // 2^e and 2^-e for a normal x = m 2^e, 1 <= |m| < 2 (e within +-1022).
@@ -185,6 +235,7 @@ __host__ __device__ inline int dc_exp(double x)
 
 // Root i of the secular equation, x_i = d[org] + mu: in (d_i, d_(i+1)), or for
 // i = K - 1 in (d_i, d_i + sum z^2].
+template <int WAY>
 __host__ __device__ inline void dc_root(const DcPoles& p, int i, const DcLanes& g, int& org, double& mu)
 {
     const int K = p.K;
@@ -200,13 +251,13 @@ __host__ __device__ inline void dc_root(const DcPoles& p, int i, const DcLanes& 
     float lo32, hi32, m32;
     if (last) {
         org = K - 1;
-        float zz = 0.0f;
-        for (int j = g.sub; j < K; j += g.P) zz += p.z2[j];
+        float zz[WAY] = {};
+        dc_each<WAY>(K, g, [&](int j, int q) { zz[q] += p.z2[j]; });
         lo32 = 0.0f;
         hi32 = g.sum(zz);
         m32 = 0.5f * hi32;
     } else {
-        const DcSums<float> s = dc_sums(p, split, i, 0.5f * gapf, g);
+        const DcSums<float> s = dc_sums<WAY>(p, split, i, 0.5f * gapf, g);
         // f(middle) >= 0: the root lies in the left half
         org = 1.0f + s.psi + s.phi >= 0.0f ? i : i + 1;
         lo32 = org == i ? 0.0f : -gapf;
@@ -214,7 +265,7 @@ __host__ __device__ inline void dc_root(const DcPoles& p, int i, const DcLanes& 
         m32 = 0.5f * (lo32 + hi32);
     }
     for (int it = 0; it < 20; ++it) {
-        const DcSums<float> s = dc_sums(p, split, org, m32, g);
+        const DcSums<float> s = dc_sums<WAY>(p, split, org, m32, g);
         const float f = 1.0f + s.psi + s.phi;
         if (f < 0.0f) lo32 = m32;
         else hi32 = m32;
@@ -233,8 +284,8 @@ __host__ __device__ inline void dc_root(const DcPoles& p, int i, const DcLanes& 
     double lo, hi;
     const double dorg = p.d[org];
     if (last) {
-        double zz = 0.0;
-        for (int j = g.sub; j < K; j += g.P) zz += p.z[j] * p.z[j];
+        double zz[WAY] = {};
+        dc_each<WAY>(K, g, [&](int j, int q) { zz[q] = fma(p.z[j], p.z[j], zz[q]); });
         lo = 0.0;
         hi = g.sum(zz) * (1.0 + 1e-12);
     } else {
@@ -246,7 +297,7 @@ __host__ __device__ inline void dc_root(const DcPoles& p, int i, const DcLanes& 
     if (!(x > lo && x < hi)) x = 0.5 * (lo + hi);
     const double di = p.d[split] - dorg, dj = p.d[split + 1] - dorg;
     for (int it = 0; it < 200; ++it) {
-        const DcSums<double> s = dc_sums(p, split, dorg, x, g);
+        const DcSums<double> s = dc_sums<WAY>(p, split, dorg, x, g);
         const double f = 1.0 + s.psi + s.phi;
         // f is known to the rounding of its terms
         if (fabs(f) <= 2.0 * kDcEps * (1.0 + fabs(s.psi) + fabs(s.phi))) break;
@@ -275,43 +326,41 @@ __host__ __device__ inline void dc_root(const DcPoles& p, int i, const DcLanes& 
 // Loewner: the z_j (up to a common factor) for which the computed roots are
 // exact: z_j^2 = (x_(K-1) - d_j) prod_(i<j) (x_i - d_j)/(d_i - d_j)
 //                                prod_(j<=i<K-1) (x_i - d_j)/(d_(i+1) - d_j).
+template <int WAY>
 __host__ __device__ inline double dc_loewner(const DcPoles& p, const int* org, const double* mu, int j,
                                              const DcLanes& g)
 {
     const double dj = p.d[j];
-    double v = 1.0;
-    for (int i = g.sub; i < p.K; i += g.P) {
+    double v[WAY];
+#pragma unroll
+    for (int q = 0; q < WAY; ++q) v[q] = 1.0;
+    dc_each<WAY>(p.K, g, [&](int i, int q) {
         const double num = (p.d[org[i]] - dj) + mu[i];
-        if (i == p.K - 1) v *= num;
-        else v *= num * dc_rcp(p.d[i < j ? i : i + 1] - dj);
-    }
-#ifdef __CUDA_ARCH__
-    for (int o = g.P >> 1; o > 0; o >>= 1) v *= __shfl_xor_sync(g.mask, v, o);
-#endif
-    return copysign(sqrt(fabs(v)), p.z[j]);
+        if (i == p.K - 1) v[q] *= num;
+        else v[q] *= num * dc_rcp(p.d[i < j ? i : i + 1] - dj);
+    });
+    return copysign(sqrt(fabs(g.product(v))), p.z[j]);
 }
 
 // First and last components of the eigenvector of root i: of the normalised
 // vector with entries zh_j / (d_j - x_i), against the rows F and L of the
 // pieces' eigenvector matrices (lst: position of pole j in F and L).
+template <int WAY>
 __host__ __device__ inline void dc_vector(const DcPoles& p, const double* zh, const double* F,
                                           const double* L, const int* lst, int org, double mu,
-                                          const DcLanes& g, double& first, double& lastc)
+                                          const DcLanes& g, bool want_last, double& first, double& lastc)
 {
     const double dorg = p.d[org];
-    double s = 0.0, a = 0.0, b = 0.0;
-    for (int j = g.sub; j < p.K; j += g.P) {
+    double s[WAY] = {}, a[WAY] = {}, b[WAY] = {};
+    dc_each<WAY>(p.K, g, [&](int j, int q) {
         const double u = zh[j] * dc_rcp((p.d[j] - dorg) - mu);
-        s += u * u;
-        a += u * F[lst[j]];
-        b += u * L[lst[j]];
-    }
-    s = g.sum(s);
-    a = g.sum(a);
-    b = g.sum(b);
-    const double inv = dc_rsqrt(s);
-    first = a * inv;
-    lastc = b * inv;
+        s[q] = fma(u, u, s[q]);
+        a[q] = fma(u, F[lst[j]], a[q]);
+        if (want_last) b[q] = fma(u, L[lst[j]], b[q]);
+    });
+    const double inv = dc_rsqrt(g.sum(s));
+    first = g.sum(a) * inv;
+    lastc = g.sum(b) * inv;
 }
 
 // Close poles of one merge, in the order of its kept list: a pair whose
@@ -391,7 +440,7 @@ __host__ __device__ inline size_t dc_smem(int k)
 __host__ __device__ inline int dc_lanes_per_root(int k, int nth)
 {
     int P = 1;
-    while (P < 4 && 2 * P * k <= nth && 2 * P <= k) P <<= 1;
+    while (P < 4 && 2 * P * k <= nth) P <<= 1;
     return P;
 }
 
@@ -529,6 +578,7 @@ struct DcLevel {
         const int b = beg(g);
         return DcPoles{w.dc + b, w.zc + b, w.hi + b, w.lo + b, w.z2 + b, kept(g)};
     }
+    template <int WAY>
     __host__ __device__ void roots(int g, const DcLanes& ln) const
     {
         const int b = beg(g), i = g - b;
@@ -536,22 +586,24 @@ struct DcLevel {
         if (i >= p.K) return;
         int org;
         double mu;
-        dc_root(p, i, ln, org, mu);
+        dc_root<WAY>(p, i, ln, org, mu);
         if (ln.sub == 0) {
             w.org[g] = org;
             w.mu[g] = mu;
         }
     }
+    template <int WAY>
     __host__ __device__ void loewner(int g, const DcLanes& ln) const
     {
         const int b = beg(g), i = g - b;
         const DcPoles p = poles(g);
         if (i >= p.K) return;
-        const double v = dc_loewner(p, w.org + b, w.mu + b, i, ln);
+        const double v = dc_loewner<WAY>(p, w.org + b, w.mu + b, i, ln);
         if (ln.sub == 0) w.zh[g] = v;
     }
     // rows of the new eigenvectors, into d, f, l: the roots first, then the
     // deflated poles, in no order yet
+    template <int WAY>
     __host__ __device__ void vectors(int g, const DcLanes& ln) const
     {
         const int b = beg(g), i = g - b;
@@ -560,7 +612,7 @@ struct DcLevel {
             double a, c;
             const int org = w.org[g];
             const double mu = w.mu[g];
-            dc_vector(p, w.zh + b, w.F, w.L, w.lst + b, org, mu, ln, a, c);
+            dc_vector<WAY>(p, w.zh + b, w.F, w.L, w.lst + b, org, mu, ln, 2 * half < k, a, c);
             if (ln.sub == 0) {
                 w.d[g] = p.d[org] + mu;
                 w.f[g] = a;
@@ -668,13 +720,13 @@ __device__ inline bool dc_solve(DcWork& w, double* e, int k, int& ex)
             __syncthreads();
         }
         if (on)
-            for (int g = grp; g < k; g += ngrp) L.roots(g, ln);
+            for (int g = grp; g < k; g += ngrp) L.roots<1>(g, ln);
         __syncthreads();
         if (on)
-            for (int g = grp; g < k; g += ngrp) L.loewner(g, ln);
+            for (int g = grp; g < k; g += ngrp) L.loewner<1>(g, ln);
         __syncthreads();
         if (on)
-            for (int g = grp; g < k; g += ngrp) L.vectors(g, ln);
+            for (int g = grp; g < k; g += ngrp) L.vectors<1>(g, ln);
         __syncthreads();
         if (on) L.order(tid, nth);
         __syncthreads();
@@ -682,6 +734,75 @@ __device__ inline bool dc_solve(DcWork& w, double* e, int k, int& ex)
         w = L.w;
     }
     return true;
+}
+
+// The same for many matrices of up to 32 rows, several in a warp (lane `base` + t: row
+// t < kmax of a matrix of k <= kmax rows, kmax the same in all lanes; k = 0: none): one
+// lane per root, which keeps apart the partial sums of the four lanes that it has
+// above, so that the bits are the same.  All 32 lanes of the warp call it.
+// For a block per matrix the scalar part of a step, which every lane repeats, and the
+// rows that fill no warp take most of the FP64 units' time once there are matrices
+// enough.  us, block per matrix | packed (64 registers, 32 warps per SM): 4096 matrices
+// k = 4 72 | 33, 8 137 | 93, 16 410 | 279, 32 1177 | 818; 16384 k = 5 509 | 157, 8 528 | 231,
+// 12 1190 | 791, 16 1449 | 858; 1024 k = 8 72 | 70, 16 132 | 125, 20 201 | 247.  (One thread
+// per matrix, evc_tridiag.cuh, with 16384: 82, 195, 406 and 699, other bits.)
+__device__ inline bool dc_solve_packed(DcWork& w, double* e, int k, int kmax, int base, int tid, int& ex)
+{
+    const unsigned group = (kmax == 32 ? 0xffffffffu : (1u << kmax) - 1u) << base;
+    int mx = -100000, bad = 0;
+    if (tid < k) {
+        const double a = fabs(w.d[tid]), b = tid + 1 < k ? fabs(e[tid]) : 0.0;
+        bad = !isfinite(a) || !isfinite(b);
+        const double m = fmax(a, b);
+        if (m > 0.0 && isfinite(m)) mx = ilogb(m) + 1;
+    }
+    ex = -100000;
+    for (int t = 0; t < kmax; ++t) ex = max(ex, __shfl_sync(0xffffffffu, mx, min(base + t, 31)));
+    if (ex == -100000) ex = 0;
+    if (__ballot_sync(0xffffffffu, bad) & group) k = 0;     // (its lanes stay for the barriers)
+    const bool ok = k > 0;
+    if (tid < k) {
+        w.d[tid] = scalbn(w.d[tid], -ex);
+        if (tid + 1 < k) e[tid] = scalbn(e[tid], -ex);
+        w.f[tid] = w.l[tid] = 1.0;
+    }
+    __syncwarp();
+    if (2 * tid < k) {
+        const int t = 2 * tid;
+        const double a = t > 0 ? fabs(e[t - 1]) : 0.0, b = t + 2 < k ? fabs(e[t + 1]) : 0.0;
+        if (t + 1 < k) dc_pair(w.d[t] - a, e[t], w.d[t + 1] - b, w.d + t, w.f + t, w.l + t);
+        else w.d[t] -= a;
+    }
+    __syncwarp();
+    const DcLanes ln{0, 1, 0};
+    for (int half = 2; half < kmax; half *= 2) {
+        DcLevel lv{w, e, k, half, 1};
+        const bool act = half < k && tid < k;
+        if (act) lv.sort(tid, kmax);
+        __syncwarp();
+        if (act) lv.flag(tid, kmax);
+        __syncwarp();
+        if (act) lv.keep(tid, kmax);
+        __syncwarp();
+        const bool close = __ballot_sync(0xffffffffu, act && lv.close(tid)) & group;
+        if (close && act && lv.beg(tid) == tid) lv.deflate_close(tid);
+        __syncwarp();
+        if (close && act) lv.keep(tid, kmax);
+        __syncwarp();
+        if (act) lv.roots<4>(tid, ln);
+        __syncwarp();
+        if (act) lv.loewner<4>(tid, ln);
+        __syncwarp();
+        if (act) lv.vectors<4>(tid, ln);
+        __syncwarp();
+        if (act) lv.order(tid, kmax);
+        __syncwarp();
+        if (half < k) {
+            lv.swap();
+            w = lv.w;
+        }
+    }
+    return ok;
 }
 
 // Sum of the squared first components over the eigenvalues below sigma, by the
@@ -695,6 +816,35 @@ __device__ inline double dc_weight_below(const DcWork& w, int k, int ex, double 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     return q;
+}
+// The same for packed matrices, in lane tid = 0: the additions of that tree whose
+// terms are not zero by their place.
+__device__ inline double dc_weight_below_packed(const DcWork& w, int k, int ex, int base, int tid, double sigma)
+{
+    double q = tid < k && w.d[tid] < scalbn(sigma, -ex) ? w.f[tid] * w.f[tid] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const double v = __shfl_sync(0xffffffffu, q, min(base + tid + o, 31));
+        if (tid < o && tid + o < k) q += v;
+    }
+    return q;
+}
+
+// Packed matrices: threads per block, matrices per block, and bytes of shared memory of
+// a matrix of up to k rows.
+constexpr int kPackedThreads = 128, kPackedBlocks = 8;   // (blocks per SM: 64 registers)
+__host__ __device__ inline bool dc_packed_pays(int k, int matrices) { return k <= 16 ? matrices >= 1024 : k <= 32 && matrices >= 4096; }
+__host__ __device__ inline int dc_packed_matrices(int k) { return kPackedThreads / 32 * (32 / k); }
+__host__ __device__ inline size_t dc_packed_bytes(int k) { return dc_smem(k) + (size_t)((k + 1) & ~1) * sizeof(double); }
+// This lane's matrix among the block's (-1: none) and its place in it.
+struct DcPlace {
+    int at, base, tid;
+};
+__device__ inline DcPlace dc_packed_place(int k)
+{
+    const int lane = threadIdx.x & 31, per = 32 / k, in = lane / k;
+    // (the lanes left over read the last matrix's lanes in the shuffles)
+    return in < per ? DcPlace{(int)(threadIdx.x >> 5) * per + in, in * k, lane - in * k} : DcPlace{-1, 0, 32};
 }
 #endif
 

@@ -783,6 +783,38 @@ __global__ void __launch_bounds__(512) quad_kernel(Run r, int i)
     }
 }
 
+// The same with several columns in a warp, for rules of up to kmax <= 32 nodes.
+__global__ void __launch_bounds__(kPackedThreads, kPackedBlocks) quad_packed_kernel(Run r, int i, int kmax)
+{
+    extern __shared__ __align__(16) unsigned char qp[];
+    const DcPlace me = dc_packed_place(kmax);
+    const int at = blockIdx.x * dc_packed_matrices(kmax) + me.at;
+    const int c = me.at >= 0 && at < r.ncol_real ? at : -1;
+    bool running = false;
+    if (r.shared) {
+        for (int s = threadIdx.x & 31; s < r.S; s += 32) running |= quad_needed(r, s, i);
+        running = __any_sync(0xffffffffu, running) && c >= 0;
+    } else {
+        running = c >= 0 && quad_needed(r, r.shift_of[c], i);
+    }
+    if (!__any_sync(0xffffffffu, running)) return;
+    const int k = !running ? 0 : r.kdone[c] ? min(r.kdone[c], i) : i;
+    const int kr = r.ga && k > 1 ? 2 * k - 1 : k;
+    double* e = reinterpret_cast<double*>(qp + max(me.at, 0) * dc_packed_bytes(kmax));
+    DcWork w = dc_carve(e + ((kmax + 1) & ~1), max(kr, 1));
+    if (running) tridiag_fill(r.alpha + c, r.beta + c, r.ncol, k, r.ga != 0, w.d, e, me.tid, kmax);
+    __syncwarp();
+    int ex;
+    const bool ok = dc_solve_packed(w, e, kr, kmax, me.base, me.tid, ex);
+    if (running && !ok && me.tid == 0) atomicExch(r.err, DERR_NUMERIC);
+    for (int s = 0; s < (r.shared ? r.S : 1); ++s) {
+        if (r.shared && r.sdone[s]) continue;
+        const double q = dc_weight_below_packed(w, ok ? kr : 0, ex, me.base, me.tid, r.shared ? r.shifts[s] : 0.0);
+        if (running && me.tid == 0 && (!r.shared || c < r.m))
+            r.quad[r.shared ? (int64_t)s * r.m + c : c] = ok ? (double)r.n * q : 0.0;
+    }
+}
+
 // Per-shift mean L_s(i) = (1/m) sum_j quad_j in a fixed tree, and the stop
 // rule: a shift stops at its last step (skmax[s]) or, under its tolerance, at
 // the first step i >= max(3, min_steps) with |L_s(i) - L_s(i-1)| <= tol and
@@ -1042,7 +1074,13 @@ cudaError_t launch_finish(const Run& r, int i, cudaStream_t st)
         const cudaError_t e = launch_arnoldi_quad(r, i, st);
         if (e != cudaSuccess) return e;
     } else {
-        quad_kernel<<<r.ncol_real, dc_threads(kr), smem, st>>>(r, i);
+        if (dc_packed_pays(kr, r.ncol_real)) {
+            const int per = dc_packed_matrices(kr);
+            quad_packed_kernel<<<(r.ncol_real + per - 1) / per, kPackedThreads, per * dc_packed_bytes(kr), st>>>(
+                r, i, kr);
+        } else {
+            quad_kernel<<<r.ncol_real, dc_threads(kr), smem, st>>>(r, i);
+        }
     }
     shift_kernel<<<r.S, kThreads, 0, st>>>(r, i);
     return cudaGetLastError();

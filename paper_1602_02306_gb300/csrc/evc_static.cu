@@ -84,6 +84,28 @@ static_quad_block_kernel(const double* alpha, const double* beta, const int* kco
     }
 }
 
+// Columns of up to 32 rows, several in a warp: the same bits.
+__global__ void __launch_bounds__(evc::kPackedThreads, evc::kPackedBlocks)
+static_quad_packed_kernel(const double* alpha, const double* beta, const int* kcol, int k, int ncol,
+                          double vnorm2, double* quad, int* status)
+{
+    extern __shared__ __align__(16) unsigned char qp[];
+    const evc::DcPlace me = evc::dc_packed_place(k);
+    const int c = me.at < 0 ? ncol : blockIdx.x * evc::dc_packed_matrices(k) + me.at;
+    const int kc = c < ncol ? (kcol ? kcol[c] : k) : 0;
+    const bool valid = kc >= 1 && kc <= k;
+    double* e = reinterpret_cast<double*>(qp + max(me.at, 0) * evc::dc_packed_bytes(k));
+    evc::DcWork w = evc::dc_carve(e + ((k + 1) & ~1), valid ? kc : 1);
+    if (valid) evc::tridiag_fill(alpha + c, beta + c, ncol, kc, false, w.d, e, me.tid, k);
+    __syncwarp();
+    int ex;
+    const bool ok = evc::dc_solve_packed(w, e, valid ? kc : 0, k, me.base, me.tid, ex);
+    const double q = evc::dc_weight_below_packed(w, ok ? kc : 0, ex, me.base, me.tid, 0.0);
+    if (me.tid != 0 || c >= ncol) return;
+    quad[c] = ok ? vnorm2 * q : CUDART_NAN;
+    if (!ok && status) atomicCAS(status, EVC_OK, valid ? EVC_ENUMERIC : EVC_EINVAL);
+}
+
 int say(char* buf, size_t len, int code, const char* msg)
 {
     if (buf && len) snprintf(buf, len, "%s", msg);
@@ -137,17 +159,26 @@ extern "C" int evc_gauss_quadrature_static(const double* d_alpha, const double* 
         }
     }
     const size_t smem = evc::dc_smem(k) + (size_t)((k + 1) & ~1) * sizeof(double);   // at most 31 KB
-    // One block per column while the columns leave FP64 units idle; with more, a
-    // thread per column does less work in all.  Measured (thread | block): 64 x
-    // k = 40 3572 | 217 us, 4096 x k = 16 694 | 426, 16384 x k = 16 701 | 1501,
-    // 8192 x k = 32 about equal (2.5 ms); 4096 x k = 4 60 | 76, 2048 x k = 4
-    // about equal.
-    if (k >= 32 || ncol <= (k > 4 ? 4096 : 2048))
-        static_quad_block_kernel<<<ncol, evc::dc_threads(k), smem, st>>>(
-            d_alpha, d_beta, d_kcol, k, ncol, vnorm2, d_quad, d_status);
-    else
+    // Divide and conquer while the columns leave FP64 units idle; with more, a thread per
+    // column does less work in all.  Measured
+    // (thread | divide and conquer): 64 x k = 40 3572 | 217 us, 4096 x k = 16 694 | 279, 16384 x
+    // k = 16 701 | 858, 16384 x k = 8 195 | 231, 8192 x k = 9 244 | 278, 8192 x k = 32 about
+    // equal (2.5 ms); 2048 x k = 4 56 | 33, 16384 x k = 4 56 | 70.  The two agree to
+    // rounding only: see the header.
+    if (k >= 32 || ncol <= (k > 4 ? 4096 : 2048)) {
+        if (evc::dc_packed_pays(k, ncol)) {
+            const int per = evc::dc_packed_matrices(k);
+            static_quad_packed_kernel<<<(ncol + per - 1) / per, evc::kPackedThreads,
+                                        per * evc::dc_packed_bytes(k), st>>>(
+                d_alpha, d_beta, d_kcol, k, ncol, vnorm2, d_quad, d_status);
+        } else {
+            static_quad_block_kernel<<<ncol, evc::dc_threads(k), smem, st>>>(
+                d_alpha, d_beta, d_kcol, k, ncol, vnorm2, d_quad, d_status);
+        }
+    } else {
         static_quad_kernel<<<(ncol + 127) / 128, 128, 0, st>>>(d_alpha, d_beta, d_kcol, k, ncol,
                                                                vnorm2, d_quad, scratch, d_status);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return say(errbuf, errlen, EVC_ECUDA, cudaGetErrorString(e));
     return EVC_OK;

@@ -40,9 +40,9 @@ extern "C" void dc_eig(int k, const double* diag, const double* off, double* the
                 if (L.beg(g) == g) L.deflate_close(g);
             L.keep(0, 1);
         }
-        for (int g = 0; g < k; ++g) L.roots(g, ln);
-        for (int g = 0; g < k; ++g) L.loewner(g, ln);
-        for (int g = 0; g < k; ++g) L.vectors(g, ln);
+        for (int g = 0; g < k; ++g) L.roots<1>(g, ln);
+        for (int g = 0; g < k; ++g) L.loewner<1>(g, ln);
+        for (int g = 0; g < k; ++g) L.vectors<1>(g, ln);
         L.order(0, 1);
         L.swap();
         w = L.w;
