@@ -485,7 +485,7 @@ void evc_server_destroy(evc_server* srv);
  * loads the library holds until the process exits.
  *
  * It computes the same quadrature as the last step of evc_count_slices
- * (Sec. 3, Eq. gauss_quad): for each column c, ||v||^2 sum over the negative
+ * (Sec. 3, Eq. gauss_quad), to rounding: for each column c, ||v||^2 sum over the negative
  * eigenvalues theta of J_kc of z(1)^2, from coefficients laid out as the
  * estimator keeps them on the device:
  *   d_alpha : double[k * ncol],     d_alpha[t*ncol + c] = alpha_{t+1}
@@ -507,11 +507,17 @@ void evc_server_destroy(evc_server* srv);
  * message in errbuf (optional host buffer of errlen bytes).
  * The first call on a device looks up the device address of the scratch
  * array (cudaGetSymbolAddress) with that device current, so make that first
- * call outside any stream capture.  Every call reuses the same array and the
- * kernel writes each scratch entry before reading it, so a previous call's
- * leftovers do not matter; but calls whose kernels can overlap on the GPU
- * (different streams without ordering between them) race on the array and
- * give wrong results -- serialise them.                                       */
+ * call outside any stream capture.
+ * Two eigensolvers take turns: the estimator's (divide and conquer, in shared
+ * memory) for k >= 32 and for up to 4096 columns (2048 for k <= 4, none for
+ * k = 3), and one thread per column (QR, in the scratch array) otherwise.  Both
+ * are within some 1e-15 ||J|| of J, so a column's result may differ in the last
+ * bits between calls on either side of that line, never between calls on one.
+ * Calls of the second kind reuse the array and the kernel writes each scratch
+ * entry before reading it, so a previous call's leftovers do not matter; but
+ * such calls whose kernels can overlap on the GPU (different streams without
+ * ordering between them) race on the array and give wrong results -- serialise
+ * them.                                                                        */
 #define EVC_STATIC_QUAD_MAX 262144
 int evc_gauss_quadrature_static(const double* d_alpha, const double* d_beta, const int* d_kcol,
                                 int k, int ncol, double vnorm2, double* d_quad, int* d_status,

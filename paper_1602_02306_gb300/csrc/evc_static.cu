@@ -160,12 +160,13 @@ extern "C" int evc_gauss_quadrature_static(const double* d_alpha, const double* 
     }
     const size_t smem = evc::dc_smem(k) + (size_t)((k + 1) & ~1) * sizeof(double);   // at most 31 KB
     // Divide and conquer while the columns leave FP64 units idle; with more, a thread per
-    // column does less work in all.  Measured
+    // column does less work in all, and for three rows, with a merge of one row, is as fast
+    // with few.  Measured
     // (thread | divide and conquer): 64 x k = 40 3572 | 217 us, 4096 x k = 16 694 | 279, 16384 x
     // k = 16 701 | 858, 16384 x k = 8 195 | 231, 8192 x k = 9 244 | 278, 8192 x k = 32 about
-    // equal (2.5 ms); 2048 x k = 4 56 | 33, 16384 x k = 4 56 | 70.  The two agree to
-    // rounding only: see the header.
-    if (k >= 32 || ncol <= (k > 4 ? 4096 : 2048)) {
+    // equal (2.5 ms); 2048 x k = 4 56 | 33, 16384 x k = 4 56 | 70; 64 to 1024 x k = 3 28 | 34.
+    // The two agree to rounding only: see the header.
+    if (k >= 32 || (k != 3 && ncol <= (k > 4 ? 4096 : 2048))) {
         if (evc::dc_packed_pays(k, ncol)) {
             const int per = evc::dc_packed_matrices(k);
             static_quad_packed_kernel<<<(ncol + per - 1) / per, evc::kPackedThreads,

@@ -1,5 +1,7 @@
 """Quadratures of many columns, several to a warp: the same bits as one block per
-column, whatever the sizes in a warp, with columns that fail among them."""
+column, whatever the sizes in a warp, with columns that fail among them; and the
+static call's two eigensolvers, which take turns by the number of columns, agree
+to rounding."""
 import numpy as np
 import pytest
 
@@ -61,6 +63,24 @@ def test_packed_columns_have_the_bits_of_single_ones(k):
     sizes[20], sizes[21] = 0, k + 1
     q, st = _static(alpha[:, 13:], beta[:, 13:], sizes[13:])
     assert st == evc.EVC_EINVAL and list(np.flatnonzero(np.isnan(q))) == [7, 8]
+
+
+@pytest.mark.parametrize("k,line", [(2, 2048), (4, 2048), (5, 4096), (16, 4096), (31, 4096)])
+def test_both_eigensolvers_agree(k, line):
+    # 0 in a gap of every spectrum: two rows of +-4 on the diagonal keep the rest away
+    rng = np.random.default_rng(k)
+    alpha = np.where(rng.random((k, line + 1)) < 0.5, -4.0, 4.0) + 0.3 * rng.standard_normal((k, line + 1))
+    beta = 0.7 + 0.6 * rng.random((k + 1, line + 1))
+    few, _ = _static(alpha[:, :line], beta[:, :line])
+    many, _ = _static(alpha, beta)
+    # both within 64 k eps ||J|| / gap of the exact weights (twice vnorm2 = 2)
+    J = np.zeros((line, k, k))
+    i = np.arange(k)
+    J[:, i, i] = alpha[:, :line].T
+    J[:, i[1:], i[:-1]] = J[:, i[:-1], i[1:]] = beta[1:k, :line].T
+    th = np.linalg.eigvalsh(J)
+    bound = 2 * 2.0 * 64 * k * EPS * np.abs(th).max(1) / np.abs(th).min(1)
+    assert np.all(np.abs(few - many[:line]) <= bound)
 
 
 @pytest.mark.parametrize("prec", [evc.EVC_FP64, evc.EVC_MIXED])
