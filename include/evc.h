@@ -251,7 +251,9 @@ int evc_get_quad_bound(evc_ctx* ctx, double* log10_bound);
  *                       batches, so a column's result is the same alone or in
  *                       a batch for one setting.
  *   EVC_OPT_STENCIL_ZB: stencil contexts: z planes per block of the stencil
- *                       pass (default 32).  Results are unchanged.
+ *                       pass (default 32); the most planes per block of the
+ *                       kernel that applies two passes at once (see
+ *                       EVC_OPT_STENCIL_PATCH).  Results are unchanged.
  *   EVC_OPT_STENCIL_PATCH: stencil contexts: points per thread of the stencil
  *                       pass, 1 (default) or 2 = a 2 x 2 patch of (x, y) points
  *                       whose inner neighbours come from registers (fewer loads
@@ -262,7 +264,13 @@ int evc_get_quad_bound(evc_ctx* ctx, double* log10_bound);
  *                       staged in shared memory by tiled tensor copies, plane
  *                       by plane (N a multiple of the tile, else 2 is used).
  *                       2 and 3 give bitwise the same results; they agree with
- *                       1 to rounding.
+ *                       1 to rounding.  The two passes of a conjugate pair of
+ *                       roots (EVC_CHEB_FACTORED, EVC_MIXED, 7-point, N even and
+ *                       at least 12) run in one kernel with tiles of its own,
+ *                       whatever this option says, with the bits of the single
+ *                       passes; only for many columns on grids of 18 to 22
+ *                       points do 2 and 3 keep the single passes, which are
+ *                       faster there.
  *   EVC_OPT_STENCIL_GROUPS: stencil contexts: 1 (default) to 4.  The stencil
  *                       passes of each step's operator application run as this
  *                       many groups of column chunks, each group on its own
@@ -376,7 +384,8 @@ int evc_get_profile(evc_ctx* ctx, evc_prof_rec* recs, int cap, int* nrec);
  * and keeps, per kernel family, the fastest of
  *   stencil pass:  z planes per block 16 / 32 / 64 (EVC_OPT_STENCIL_ZB) times
  *                  points per thread 1 / 2x2 / 2x2 in tensor-copied tiles
- *                  (EVC_OPT_STENCIL_PATCH), then
+ *                  (EVC_OPT_STENCIL_PATCH; under the Chebyshev preconditioner
+ *                  mostly those of the passes that do not run in pairs), then
  *                  1 / 2 / 4 concurrent chunk groups (EVC_OPT_STENCIL_GROUPS), and
  *                  the shapes once more if the groups changed,
  *   CSR pass:      threads per block 128 / 256 / 512 (EVC_OPT_CSR_THREADS),

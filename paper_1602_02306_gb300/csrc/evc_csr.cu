@@ -220,10 +220,11 @@ csr_pass_kernel(CArgs a)
 // of q_i.  Same ownership, same order of the sums and same roundings as above.
 // Bound by the latency of the gathers (128 or 256 bytes at random from L2 and
 // DRAM): all eight of a batch are in flight, the next batch of (col, val) pairs
-// is fetched meanwhile, and what the pass touches once leaves L2 first.  At least
-// 36 warps per SM: the registers that this leaves (56) hold the batch, and the
-// time no longer depends on the block size (two gathers in flight: 30 % slower;
-// eight without the bound: 1.18, 1.51 and 1.73 ms with 128, 64 and 256 threads).
+// is fetched meanwhile, and what the pass touches once leaves L2 first.  The bound
+// on the registers (56 and 36 warps per SM with 128 threads, 64 and 32 with 256 and
+// 512, whose blocks come in fours and twos) holds the batch (two gathers in flight:
+// 30 % slower; eight without the bound: 1.18, 1.51 and 1.73 ms with 128, 64 and 256
+// threads; with it 1.01 and 1.06 with 128 and 256).
 // FP32 rows are padded to whole batches (their own row of x, times zero): smaller
 // batches for the rest cost more than the gathers they save (2M rows, six passes:
 // 25.5 | 26.2 to 27.0 ms).  FP64 rows are not: a padded entry takes the FP64 units,
@@ -234,9 +235,8 @@ csr_pass_kernel(CArgs a)
 //   kernel that writes the copy, 600k 1.66 | 1.10, 30k (one row of 2000 entries
 //   is the critical path) 0.55 | 0.21; FP64 Jacobi 200k 2.49 | 1.42 (FP64 units:
 //   one operation per entry and column, before two).
-// 2M rows read 0.5 GB of structure and about 5 GB of x rows per chunk from DRAM
-// (the 256 MB of a chunk's x are twice L2) at 5 TB/s: what random 128-byte reads
-// reach there.  Slices of 16 or 8 columns of x, which fit L2, are no way out: 64
+// 2M rows move 6.8 GB per chunk through DRAM (the 256 MB of a chunk's x are twice L2)
+// at 6.25 TB/s, 0.92 of the copy peak: hits in L2 not counted, which make it 7.2.  Slices of 16 or 8 columns of x, which fit L2, are no way out: 64
 // and 32-byte gathers took 6.5 and 10.7 ms per pass.
 template <typename T, int PM, int NT, bool PRE>
 __global__ void __launch_bounds__(NT, 36 * 32 / NT)

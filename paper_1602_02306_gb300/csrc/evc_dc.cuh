@@ -1,6 +1,7 @@
 // evc_dc.cuh -- eigenvalues and first eigenvector components of a symmetric
 // tridiagonal J_k (the nodes and weights of Sec. 3, Eq. gauss_quad) by Cuppen's
-// divide and conquer, one thread block per matrix.
+// divide and conquer, one thread block per matrix or, for many short ones, several
+// matrices per warp.  (Also compiled by the host compiler, which tests the phases.)
 //
 // J is cut into pieces of two rows by subtracting |beta| from both diagonal
 // entries at every cut; pieces are merged pairwise.  A merge of two solved pieces is
@@ -22,13 +23,15 @@
 // What bounds it: FP64 instructions.  One of a warp holds its scheduler's FP64
 // unit for tens of cycles however few lanes are active, so the QR iteration of
 // evc_tridiag.cuh -- a serial chain of about 0.85 k^2 rotations of some 45 of
-// them -- took 2.3 ms at k = 40 and 22 ms at k = 134 on one thread per column.
+// them -- took a count, which kept its scratch in shared memory, 2.3 ms at k = 40
+// and 22 ms at k = 134 on one thread per column.
 // Here the lanes of a block share the roots (P lanes per root, each summing
 // every P-th term), and a root is first brought to FP32 accuracy in FP32 --
 // its starting point only -- after which two FP64 evaluations suffice.
-// Measured, 64 columns (QR | this): k = 8 175 | 69 us, 40 3572 | 217 us,
-// 134 36.2 | 1.03 ms, 256 137 | 2.1 ms; 4096 columns: k = 8 198 | 142 us,
-// 40 3.83 | 2.23 ms.  Errors against LAPACK: the same 1e-15 (QR's too).
+// Measured in the static call, whose QR has its scratch in global memory, 64
+// columns (QR | this): k = 8 175 | 68 us, 40 3572 | 209 us, 134 36.2 | 1.0 ms, 256
+// 137 | 2.1 ms; 4096 columns: k = 8 194 | 93 us, 16 690 | 279 us, 40 3.83 | 2.2 ms.
+// Errors against LAPACK: the same 1e-15 (QR's too).
 #pragma once
 
 #include <cmath>
@@ -93,7 +96,8 @@ __host__ __device__ inline void dc_each(int K, const DcLanes& g, F&& term)
 }
 
 // 1/x to working precision: the hardware's approximation (20 bits) and two
-// Newton steps.  x is a difference of distinct poles or of a pole and a root.
+// Newton steps, each of which squares the relative error: 2^-40, then the rounding
+// of the last step, below 2 ulp.  x is a difference of distinct poles or of a pole and a root.
 __host__ __device__ inline double dc_rcp(double x)
 {
 #ifdef __CUDA_ARCH__
@@ -698,7 +702,7 @@ __device__ inline bool dc_solve(DcWork& w, double* e, int k, int& ex)
     __syncthreads();
     const int P = dc_lanes_per_root(k, nth);
     const int grp = tid / P, ngrp = nth / P;
-    const DcLanes ln{tid % P, P, P == 32 ? 0xffffffffu : ((1u << P) - 1u) << ((tid & 31) & ~(P - 1))};
+    const DcLanes ln{tid % P, P, ((1u << P) - 1u) << ((tid & 31) & ~(P - 1))};
     const bool on = tid < nth;
     for (int half = 2; half < k; half *= 2) {
         DcLevel L{w, e, k, half, P};

@@ -29,7 +29,8 @@
 // one pass.  The Gram row of q_i is formed in the same sweep as Q_i^T w.
 //
 // Reductions are deterministic: per-thread partial sums over a fixed row
-// set (FP32 runs of 16 rows promoted to FP64 in mixed mode), a fixed
+// set (FP32 runs of one tile, 32 rows in the dot kernel and 8 per warp in the
+// update's norm, promoted to FP64 in mixed mode), a fixed
 // shared-memory tree, then a fixed-order sum over row blocks.  A column's
 // result does not depend on which other columns share the launch.
 #include "evc_internal.cuh"

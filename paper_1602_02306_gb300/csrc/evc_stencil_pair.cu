@@ -323,6 +323,10 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
                     if (live) sts(u0, un + uat(q, b), up[p]);
                 }
             }
+            // (No proxy fence before the stage of plane j is refilled, as the reorthogonalisation
+            // kernels have: every value read from it has gone into a u stored above, so the
+            // reads are complete.  A read whose value is used later would need one: 1 % of a
+            // Chebyshev count.)
             __syncwarp();
             if (l32 == 0) mbar_arrive(&udone[s & 1]);
             if (j >= 1) {
