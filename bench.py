@@ -329,6 +329,8 @@ def _measure(evc, W, args, stream, peak, peak_kind, steps, warmup, seed, tune=Tr
             W.N % 2 == 0 and W.N >= 12 and not _CHEB_FORM[0]:
         sname = "stencil_pair_kernel"
     roof, per_kind = _roofline(evc, recs, peak, peak_kind, sname, W)
+    if roof and roof["kernel"] == "stencil_pair_kernel":
+        roof["class_note"] = "the class also holds the single (H - sigma) pass of each step"
     psteps = float(m * int(np.sum(st)))
     return ctx, {"ms": ms, "L": L, "steps_used": st, "quad": q, "clocks": clk, "roofline": roof,
                  "quad_bound": qbound,
