@@ -1034,7 +1034,7 @@ cudaError_t launch_update_w(const Run& r, int i, cudaStream_t st)
     // 128 columns: 28.3 -> 24.4 ms per 30 steps; FP64, 200k rows, 80 columns: 47.2 ->
     // 32.3 ms per 40 steps).  A block's start counts as half a tile (1024 rows, 8192
     // columns, FP32, 30 steps: one block 4.2, two 5.2 ms).  Below one block per SM a block
-    // has the SM to itself and takes some 0.65 of the time (FP64 and T^-1 0.7, and 0.6
+    // has the SM to itself and takes some 0.65 of the time (T^-1 0.75; FP64 0.7, and 0.6
     // where it fills all SMs; 262k rows, 64 columns, FP64: one block 18.5, three 19.5 ms;
     // 200k rows: 16.9, 14.8).
     // (One resident block per SM where a late step's coefficients leave room for no
@@ -1042,7 +1042,7 @@ cudaError_t launch_update_w(const Run& r, int i, cudaStream_t st)
     const size_t smem = update_smem<T>(i);
     const int per_sm = smem > 112 * 1024 ? 1 : 2, slots = 152 * per_sm, blocks = r.nblk * r.nchunk;
     const int64_t tiles = ((r.n + r.nblk - 1) / r.nblk + update_rows(sizeof(T)) - 1) / update_rows(sizeof(T));
-    const double alone = sizeof(T) == 4 && !TW ? 0.65 : blocks > 144 ? 0.6 : 0.7;
+    const double alone = sizeof(T) == 4 ? (TW ? 0.75 : 0.65) : blocks > 144 ? 0.6 : 0.7;
     auto cost = [&](int p) {
         const int64_t b = (int64_t)blocks * p;
         const double rounds = per_sm == 2 && b <= 152 ? alone : (double)((b + slots - 1) / slots);
