@@ -188,12 +188,13 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
     const uint32_t xbase = smem_addr(raw), ubase = xbase + LA * G::XB;
     __shared__ uint64_t full[LA];            // a plane of x has landed
     __shared__ uint64_t udone[2];            // every warp has stored its u of a plane (and read x for it)
-    __shared__ int s_fail, s_last[G::BOXES];
+    __shared__ int s_fail, s_last[G::BOXES];   // ... and the last plane that a box was issued of
     __shared__ int4 boxes[G::BOXES];
     if (threadIdx.x == 0) {
         for (int s = 0; s < LA; ++s) mbar_init(&full[s], G::BOXES);
         for (int s = 0; s < 2; ++s) mbar_init(&udone[s], NCW);
         s_fail = 0;
+        for (int b = 0; b < G::BOXES; ++b) s_last[b] = -1;
         mbar_init_fence();
     }
     const int N = a.N;
@@ -224,7 +225,6 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
     }
     __syncthreads();
     const int pts = warp < 2 ? TS * G::H : warp < 4 ? 2 * TS : warp < 8 ? 2 * G::H : 1;    // of this warp's box
-    int last = -1;                           // last plane that this warp issued its box of
     auto issue = [&](int t, int stage) {
         if (warp >= G::BOXES || t >= nplane || l32 != 0 || *fail || (t >= a.have && warp == 0)) return;
         uint64_t* bar = &full[stage];
@@ -233,7 +233,7 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
         const int4 e = boxes[warp];
         mbar_arrive_expect_tx(bar, pts * NC * 4);
         load5(xbase + stage * G::XB + e.w * NC * 4, &maps.box[e.x], grp * NC, e.y & 1, e.y >> 1, z * N + e.z, ch, bar);
-        last = t;
+        s_last[warp] = t;
     };
 #pragma unroll
     for (int t = 0; t < LA; ++t) issue(t, t);
@@ -380,8 +380,6 @@ stencil_pair_kernel(const __grid_constant__ PairMaps maps, const PairArgs a)
     // plane was issued only once every warp had seen the one before it in its stage,
     // so the last LA planes are the ones that can be in flight.
     if (*fail) {
-        if (l32 == 0 && warp < G::BOXES) s_last[warp] = last;
-        __syncthreads();
         if (threadIdx.x == 0) {
             atomicCAS(a.err, DERR_NONE, DERR_TIMEOUT);
             int most = -1;
